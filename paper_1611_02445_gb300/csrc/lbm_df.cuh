@@ -239,6 +239,23 @@ LBM_DF_HD int64_t fix_from_double_cvt(double d) {
 #endif
 }
 
+// x * 2^-58 as the nearest double (ties to even), with integer instructions only: GB300 runs
+// the 64-bit integer to FP64 conversion on its 2-lane FP64 pipe.
+LBM_DF_HD double fix_to_double(int64_t x) {
+    const uint64_t a = x < 0 ? 0ull - (uint64_t)x : (uint64_t)x;
+#if defined(__CUDA_ARCH__)
+    const int n = __clzll((long long)a);
+#else
+    const int n = a ? __builtin_clzll(a) : 64;
+#endif
+    const uint64_t m = a << (n & 63);                  // leading bit at 63
+    const uint64_t k = m >> 11;                        // 53 bits; the 11 below round
+    const uint64_t up = (m & 0x7ffull) + (k & 1ull) > 0x400ull ? 1ull : 0ull;
+    // the hidden bit of k adds one to the exponent field, a carry out of k another
+    const uint64_t b = ((uint64_t)(1023 + 63 - FIX_SHIFT - 1 - n) << 52) + k + up;
+    return double_of((a ? b : 0ull) | ((uint64_t)(x < 0) << 63));
+}
+
 // Double-float of x * 2^-58 (relative error below 2^-48), from three pieces that each
 // convert to FP32 exactly: x = t 2^41 + r1 2^18 + r0 with t = floor(x / 2^41) (|t| <= 2^22),
 // 0 <= r1 < 2^23 and 0 <= r0 < 2^18. A piece p becomes a float by the 2^23 magic-number

@@ -351,90 +351,145 @@ cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]) {
 }
 
 // ----------------------------------------------------------------------------------
-// FP64 mass and momentum: per-thread FP64 partials -> warp shuffle tree -> one partial
-// per block -> a fixed-order single-block pass. No atomics, so the result depends only
-// on the launch shape, which is fixed per context.
-constexpr int RED_THREADS = 256;
+// Moments of the stored populations: the FP64 invariants (k_reduce) and the macroscopic
+// export (k_macro). Both walk the work groups, one thread per non-solid node: the loads of
+// a direction are one contiguous run of a data block and no lane idles on a solid slot.
+// GB300 runs FP64, and every conversion from or to it, on 2 lanes per SM, so the moments are
+// formed with integer (FP64 storage) or FP32 (the other formats) instructions, and FP64 is
+// left for what needs it. Measured against one thread per tile slot with FP64 moments and
+// divisions: k_reduce<F64> 103 -> 45 us on a 160^3 pack (1.4 M nodes, 219 MB: 4.9 TB/s);
+// reduction and FP64 fields together 322 -> 161 us there; the FP32 fields of a 256^3 pack
+// (5.9 M nodes) 640 us less. k_macro<F32, float> issues 65 % of cycles (the TwoSums).
+constexpr int MOM_THREADS = GROUP_LANES;   // one thread per lane of a work group
+static_assert(GROUP_MAX_NODES == MOM_THREADS && GROUP_MAX_NODES_F64 == MOM_THREADS, "one thread per lane");
 
-// Moments of one node as doubles: rho (or rho - 1 for the shifted formats, whose f is w + h
-// with sum w = 1) and j. FP64 storage: exact sums of the values in 64-bit fixed point
-// (2^-58), rounded once. FP32 / FP16 storage: the h values are FP32 numbers, summed with
-// Knuth's TwoSum so that each moment is the rounded pair hi + lo (relative error ~2^-48).
-// Either way each moment costs one or two FP64 operations, not 19: FP64 runs on 2 lanes
-// per SM.
-__device__ __forceinline__ float red_add(float a, float b, float& err) {
-    const float sum = __fadd_rn(a, b);
-    const float bb = __fsub_rn(sum, a);
-    err = __fadd_rn(err, __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
-    return sum;
+// FP64 storage: exact moments in 64-bit fixed point (2^-58). The integer conversion of a
+// population in [2^-6, 16) is exact; a node with any other value converts all 19 again with
+// the general routine (round to nearest), reading them once more in a rolled loop, so that
+// this rare path holds no registers of the common one. That routine maps NaN and Inf to
+// finite integers, so a non-finite population is found on its exponent bits and makes every
+// moment of the node NaN (what the mass watchdog of lbm_reduce looks for).
+struct FixMoments {
+    int64_t r, j[3];
+    bool nonfinite;
+};
+__device__ __forceinline__ FixMoments fix_node_moments(const double* __restrict__ f) {
+    FixMoments m;
+    m.nonfinite = false;
+    bool bad = false;
+    int64_t q[Q];
+#pragma unroll
+    for (int i = 0; i < Q; i++) q[i] = fix_from_double_fast(f[i * GROUP_LANES], bad);
+    fix_moments(q, m.r, m.j[0], m.j[1], m.j[2]);
+    if (bad) {
+        m.r = m.j[0] = m.j[1] = m.j[2] = 0;
+#pragma unroll 1
+        for (int i = 0; i < Q; i++) {
+            const double v = f[i * GROUP_LANES];
+            m.nonfinite |= (~bits_of(v) & 0x7ff0000000000000ull) == 0;
+            const int64_t w = fix_from_double(v);
+            m.r += w;
+            m.j[0] += cx(i) * w;
+            m.j[1] += cy(i) * w;
+            m.j[2] += cz(i) * w;
+        }
+    }
+    return m;
+}
+// FP32 and FP16 storage: the h values are FP32 numbers; each moment (rho - 1, j) is summed
+// with Knuth's TwoSum into a running sum and the sum of its rounding errors, so a moment is
+// the pair s + e (relative error about 2^-48).
+struct PairMoments {
+    float s[4], e[4];
+    __device__ __forceinline__ void add(int c, float v) {
+        const dfl t = two_sum(s[c], v);
+        s[c] = t.h;
+        e[c] = __fadd_rn(e[c], t.l);
+    }
+};
+template <int DT>
+__device__ __forceinline__ void add_node_moments(const typename Store<DT>::T* __restrict__ f, PairMoments& m) {
+    float h[Q];
+#pragma unroll
+    for (int i = 0; i < Q; i++) h[i] = to_arith<DT>(f[i * GROUP_LANES], i);
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        m.add(0, h[i]);
+        if (cx(i)) m.add(1, cx(i) > 0 ? h[i] : -h[i]);
+        if (cy(i)) m.add(2, cy(i) > 0 ? h[i] : -h[i]);
+        if (cz(i)) m.add(3, cz(i) > 0 ? h[i] : -h[i]);
+    }
 }
 
+// FP64 mass and momentum. Per thread: FP64 storage adds its nodes' fixed-point moments in
+// 128-bit integers (exact), the other formats add pairs in FP32 and flush them into FP64
+// sums every RED_FLUSH nodes (before the rounding errors of the error sums matter); then a
+// warp shuffle tree, one partial per block and a fixed-order single-block pass. No atomics,
+// so the result depends only on the launch shape, which is fixed per context. The half
+// force is subtracted once per thread for a uniform force, and summed per node for a field.
+constexpr int RED_THREADS = MOM_THREADS;
+constexpr int RED_FLUSH = 4;
+
+// resident CTAs per SM, and the grid: the 128-bit sums of FP64 storage need the registers
+template <int DT> constexpr int red_ctas() { return DT == LBM_F64 ? 3 : 4; }
+
 template <int DT>
-__device__ __forceinline__ void node_moments(const typename Store<DT>::T* __restrict__ f, uint32_t P, double m[4]) {
+__global__ void __launch_bounds__(RED_THREADS, red_ctas<DT>()) k_reduce(const typename Store<DT>::T* __restrict__ f,
+                                                        const int4* __restrict__ groups,
+                                                        const typename Store<DT>::R* __restrict__ gfield_c,
+                                                        int64_t n_groups, StepParams p,
+                                                        double* __restrict__ partials) {
+    const int t = threadIdx.x;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, fx = 0.0;
+    int64_t nodes = 0;
     if constexpr (DT == LBM_F64) {
-        // exact fixed-point sums; the conversion maps NaN and Inf to finite integers, so
-        // a non-finite population is tested for on its exponent bits and makes every
-        // moment of the node NaN (what the mass watchdog of lbm_reduce looks for)
-        int64_t r = 0, jx = 0, jy = 0, jz = 0;
-        uint64_t nonfinite = 0;
-#pragma unroll
-        for (int i = 0; i < Q; i++) {
-            const double v = f[data_index(P, i)];
-            const uint64_t b = (uint64_t)__double_as_longlong(v);
-            nonfinite |= (~b & 0x7ff0000000000000ull) == 0 ? 1ull : 0ull;
-            const int64_t q = fix_from_double(v);
-            r += q;
-            if (cx(i)) jx += cx(i) > 0 ? q : -q;
-            if (cy(i)) jy += cy(i) > 0 ? q : -q;
-            if (cz(i)) jz += cz(i) > 0 ? q : -q;
+        __int128 sum[4] = {0, 0, 0, 0};
+        bool nonfinite = false;
+        for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
+            const int4 h = groups[g];
+            if (t >= h.w) continue;
+            const FixMoments m = fix_node_moments(f + (p.sg0 + g) * (Q * GROUP_LANES) + t);
+            sum[0] += m.r;
+            for (int a = 0; a < 3; a++) sum[1 + a] += m.j[a];
+            nonfinite |= m.nonfinite;
+            if (gfield_c) fx += gfield_c[h.z + t];
+            nodes++;
         }
-        const double sc = 1.0 / (double)(1ull << FIX_SHIFT);
-        const double nan = __longlong_as_double(0x7ff8000000000000ll);
-        m[0] = nonfinite ? nan : __ll2double_rn(r) * sc;
-        m[1] = nonfinite ? nan : __ll2double_rn(jx) * sc;
-        m[2] = nonfinite ? nan : __ll2double_rn(jy) * sc;
-        m[3] = nonfinite ? nan : __ll2double_rn(jz) * sc;
+        for (int c = 0; c < 4; c++) {
+            // of the magnitude, so that a small negative sum has no large low word
+            const bool neg = sum[c] < 0;
+            const unsigned __int128 a = neg ? -(unsigned __int128)sum[c] : (unsigned __int128)sum[c];
+            const double hi = __ull2double_rn((uint64_t)(a >> 64)), lo = __ull2double_rn((uint64_t)a);
+            const double v = __fma_rn(hi, 18446744073709551616.0, lo) * (1.0 / (double)(1ull << FIX_SHIFT));
+            acc[c] = nonfinite ? __longlong_as_double(0x7ff8000000000000ll) : neg ? -v : v;
+        }
     } else {
-        float r = 0.f, jx = 0.f, jy = 0.f, jz = 0.f, er = 0.f, ex = 0.f, ey = 0.f, ez = 0.f;
-#pragma unroll
-        for (int i = 0; i < Q; i++) {
-            const float h = to_arith<DT>(f[data_index(P, i)], i);
-            r = red_add(r, h, er);
-            if (cx(i)) jx = red_add(jx, cx(i) > 0 ? h : -h, ex);
-            if (cy(i)) jy = red_add(jy, cy(i) > 0 ? h : -h, ey);
-            if (cz(i)) jz = red_add(jz, cz(i) > 0 ? h : -h, ez);
+        PairMoments m = {};
+        int held = 0;
+        auto flush = [&]() {
+            for (int c = 0; c < 4; c++) {
+                acc[c] += (double)m.s[c];
+                acc[c] += (double)m.e[c];
+            }
+            m = {};
+            held = 0;
+        };
+        for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
+            const int4 h = groups[g];
+            if (t >= h.w) continue;
+            add_node_moments<DT>(f + (p.sg0 + g) * (Q * GROUP_LANES) + t, m);
+            if (++held == RED_FLUSH) flush();
+            if (gfield_c) fx += (double)gfield_c[h.z + t];
+            nodes++;
         }
-        m[0] = 1.0 + ((double)r + (double)er);
-        m[1] = (double)jx + (double)ex;
-        m[2] = (double)jy + (double)ey;
-        m[3] = (double)jz + (double)ez;
+        flush();
+        acc[0] += (double)nodes;   // rho = 1 + sum h
     }
-}
-
-template <int DT>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce(const typename Store<DT>::T* __restrict__ f,
-                                                        const uint64_t* __restrict__ smask,
-                                                        const int32_t* __restrict__ tlane,
-                                                        const void* __restrict__ gfield, int64_t n_tiles,
-                                                        StepParams p, double* __restrict__ partials) {
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    const int64_t n = n_tiles * SLOTS;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = idx >> 6;
-        const int s = (int)(idx & 63);
-        const uint64_t sm = smask[k];
-        if ((sm >> s) & 1) continue;
-        double m[4];
-        node_moments<DT>(f, node_lane((uint32_t)tlane[k], sm, s), m);
-        const double Fx = gfield ? gfield_at<DT>(gfield, idx) : p.g[0];
-        acc[0] += m[0];
-        acc[1] += m[1] - 0.5 * Fx;
-        acc[2] += m[2] - 0.5 * p.g[1];
-        acc[3] += m[3] - 0.5 * p.g[2];
-    }
+    acc[1] -= 0.5 * (gfield_c ? fx : (double)nodes * p.g[0]);
+    acc[2] -= 0.5 * ((double)nodes * p.g[1]);
+    acc[3] -= 0.5 * ((double)nodes * p.g[2]);
     __shared__ double sh[RED_THREADS / 32][4];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = t & 31, warp = t >> 5;
 #pragma unroll
     for (int c = 0; c < 4; c++) {
         double v = acc[c];
@@ -443,128 +498,207 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce(const typename Store<DT>
         if (lane == 0) sh[warp][c] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (t < 4) {
         double v = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; w++) v += sh[w][threadIdx.x];
-        partials[blockIdx.x * 4 + threadIdx.x] = v;
+        for (int w = 0; w < RED_THREADS / 32; w++) v += sh[w][t];
+        partials[blockIdx.x * 4 + t] = v;
     }
 }
 
+// Fixed-order sum of the blocks' partials: 64 threads per component add every 64th partial,
+// then a shuffle tree over the eight of a warp and the eight warps in order.
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __restrict__ partials, int nb,
                                                               double* __restrict__ out) {
-    __shared__ double sh[RED_THREADS][4];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nb; b += RED_THREADS)
-        for (int c = 0; c < 4; c++) acc[c] += partials[b * 4 + c];
-    for (int c = 0; c < 4; c++) sh[threadIdx.x][c] = acc[c];
+    __shared__ double sh[RED_THREADS / 32][4];
+    const int c = threadIdx.x & 3;
+    double v = 0.0;
+    for (int b = threadIdx.x >> 2; b < nb; b += RED_THREADS / 4) v += partials[b * 4 + c];
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) < 4) sh[threadIdx.x >> 5][c] = v;
     __syncthreads();
-    for (int h = RED_THREADS / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-            for (int c = 0; c < 4; c++) sh[threadIdx.x][c] += sh[threadIdx.x + h][c];
-        __syncthreads();
+    if (threadIdx.x < 4) {
+        double s = 0.0;
+        for (int w = 0; w < RED_THREADS / 32; w++) s += sh[w][threadIdx.x];
+        out[threadIdx.x] = s;
     }
-    if (threadIdx.x < 4) out[threadIdx.x] = sh[0][threadIdx.x];
 }
 
 int reduce_blocks(int64_t n_tiles) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((n_tiles * SLOTS + RED_THREADS - 1) / RED_THREADS, 152 * 4));
 }
 
-// The own tiles of a context (all of them, or a slab context's without its ghost planes)
-// as pointers to their first tile: populations, masks, tile indices and per-slot force.
-struct OwnTiles {
-    const void* f;
-    const uint64_t* smask;
-    const int32_t* tlane;
-    const uint32_t* non_empty;
-    const void* gfield;
-    int64_t n;
-};
-static OwnTiles own_tiles(const lbm_ctx* c) {
-    const int64_t k0 = c->own_k0;
-    const size_t gsize = c->dtype == LBM_F64 ? 8 : 4;
-    return {c->f[c->cur], c->smask + k0, c->tlane + k0, c->non_empty + k0, c->gfield ? static_cast<const char*>(c->gfield) + (size_t)k0 * SLOTS * gsize : nullptr,
-            c->own_k1 - k0};
+// The per-node force in group order, if one is set.
+template <int DT> static const typename Store<DT>::R* force_c(const lbm_ctx* c) {
+    return c->gfield ? static_cast<const typename Store<DT>::R*>(c->gfield_c) : nullptr;
+}
+
+template <int DT> static int reduce_dt(lbm_ctx* c) {
+    const int64_t fits = std::min<int64_t>(c->n_partials, 152 * red_ctas<DT>());
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(fits, c->n_groups));
+    k_reduce<DT><<<nb, RED_THREADS, 0, c->stream>>>(static_cast<const typename Store<DT>::T*>(c->f[c->cur]), c->groups,
+                                                    force_c<DT>(c), c->n_groups, c->p, c->partials);
+    return nb;
 }
 
 cudaError_t launch_reduce(lbm_ctx* c, double* d_out) {
-    const int nb = c->n_partials;
-    const OwnTiles o = own_tiles(c);
-    switch (c->dtype) {
-        case LBM_F64:
-            k_reduce<LBM_F64><<<nb, RED_THREADS, 0, c->stream>>>((const double*)o.f, o.smask, o.tlane, o.gfield, o.n, c->p,
-                                                                 c->partials);
-            break;
-        case LBM_F32:
-            k_reduce<LBM_F32><<<nb, RED_THREADS, 0, c->stream>>>((const float*)o.f, o.smask, o.tlane, o.gfield, o.n, c->p,
-                                                                 c->partials);
-            break;
-        default:
-            k_reduce<LBM_F16S><<<nb, RED_THREADS, 0, c->stream>>>((const __half*)o.f, o.smask, o.tlane, o.gfield, o.n, c->p,
-                                                                  c->partials);
-    }
+    const int nb = c->dtype == LBM_F64 ? reduce_dt<LBM_F64>(c) : c->dtype == LBM_F32 ? reduce_dt<LBM_F32>(c)
+                                                                                     : reduce_dt<LBM_F16S>(c);
     k_reduce_final<<<1, RED_THREADS, 0, c->stream>>>(c->partials, nb, d_out);
     return cudaGetLastError();
 }
 
-// ----------------------------------------------------------------------------------
 // Macroscopic export from the stored post-collision populations: rho = sum f*,
 // u = (sum c f* - F/2)/rho (Eq. 5; Eq. 6 without the division for the incompressible
 // model), into dense arrays (already zeroed by the caller).
+//
+// x / r from ir, 1/r to 2^-46 or better: one Newton correction of x ir, which rounds like
+// the division (to half an ulp and a little) in three FP64 operations, where a division takes
+// about ten and a reciprocal as many.
+__device__ __forceinline__ double div_by(double x, double r, double ir) {
+    const double q = __dmul_rn(x, ir);
+    return __fma_rn(__fma_rn(-q, r, x), ir, q);
+}
+// The same in pairs for an FP32 result.
+__device__ __forceinline__ float pair_value(dfl x) { return __fadd_rn(x.h, x.l); }
+
+// What one node exports, from its exact moments (double) or from pairs (float).
+template <typename O> struct NodeFields {
+    O rho, u[3];
+};
+__device__ __forceinline__ NodeFields<double> fields_of(const double m[4], const double half[3], bool inc) {
+    NodeFields<double> o;
+    o.rho = m[0];
+    for (int a = 0; a < 3; a++) o.u[a] = inc ? m[1 + a] - half[a] : (m[1 + a] - half[a]) / m[0];
+    return o;
+}
+// FP64 results of FP64 storage for a density in [5/8, 7/4): 1/rho in pairs, widened with integer
+// instructions, so that FP64 is left with the force and three operations per component.
+__device__ __forceinline__ NodeFields<double> fields_of(const FixMoments& m, const double half[3], bool inc, bool& ok) {
+    NodeFields<double> o;
+    ok = !m.nonfinite && m.r >= (5ll << (FIX_SHIFT - 3)) && m.r < (7ll << (FIX_SHIFT - 2));
+    o.rho = fix_to_double(m.r);
+    const double ir = df_to_double_pos(df_recip(df_from_fix(m.r)));
+    for (int a = 0; a < 3; a++) {
+        double x = fix_to_double(m.j[a]);
+        if (half[a] != 0.0) x -= half[a];
+        o.u[a] = inc ? x : div_by(x, o.rho, ir);
+    }
+    return o;
+}
+// Valid for a density in [2^-20, 2^20]; `ok` says whether the result can be used.
+__device__ __forceinline__ NodeFields<float> fields_of(const dfl r, const dfl j[3], const dfl half[3], bool inc, bool& ok) {
+    NodeFields<float> o;
+    o.rho = pair_value(r);
+    ok = o.rho >= 0x1p-20f && o.rho <= 0x1p20f;
+    const dfl ir = df_recip(r);
+    for (int a = 0; a < 3; a++) {
+        const dfl x = df_sub(j[a], half[a]);
+        o.u[a] = pair_value(inc ? x : df_mul(x, ir));
+        ok = ok && fabsf(o.u[a]) <= 0x1p20f;   // false for NaN
+    }
+    return o;
+}
+
 template <int DT, typename O>
-__global__ void k_macro(const typename Store<DT>::T* __restrict__ f, const uint64_t* __restrict__ smask,
-                        const int32_t* __restrict__ tlane, const uint32_t* __restrict__ non_empty,
-                        const void* __restrict__ gfield,
-                        int64_t n_tiles, int nx, int ny, int nz, int Tx, int Ty, StepParams p,
-                        O* __restrict__ rho, O* __restrict__ u) {
-    const int64_t n = n_tiles * SLOTS;
+__global__ void __launch_bounds__(MOM_THREADS, 4) k_macro(const typename Store<DT>::T* __restrict__ f,
+                                                       const int4* __restrict__ groups,
+                                                       const uint32_t* __restrict__ fidx,
+                                                       const uint32_t* __restrict__ non_empty,
+                                                       const typename Store<DT>::R* __restrict__ gfield_c,
+                                                       int64_t n_groups, int nx, int ny, int nz, int Tx, int Ty,
+                                                       StepParams p, O* __restrict__ rho, O* __restrict__ u) {
     const int64_t N = (int64_t)nx * ny * nz;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = idx >> 6;
-        const int s = (int)(idx & 63);
-        const uint64_t sm = smask[k];
-        if ((sm >> s) & 1) continue;
-        const uint32_t t = non_empty[k];
-        const int x = TILE * (int)(t % (uint32_t)Tx) + (s & 3);
-        const int y = TILE * (int)((t / (uint32_t)Tx) % (uint32_t)Ty) + ((s >> 2) & 3);
-        const int z = TILE * (int)(t / ((uint32_t)Tx * (uint32_t)Ty)) + (s >> 4);
-        const int64_t node = x + (int64_t)nx * (y + (int64_t)ny * z);
-        double m[4];
-        node_moments<DT>(f, node_lane((uint32_t)tlane[k], sm, s), m);
-        const double r = m[0], jx = m[1], jy = m[2], jz = m[3];
-        const double Fx = gfield ? gfield_at<DT>(gfield, idx) : p.g[0];
-        rho[node] = (O)r;
-        if (p.eq == LBM_EQ_INCOMPR) {
-            // Eq. 6: no division by the density
-            u[node] = (O)(jx - 0.5 * Fx);
-            u[N + node] = (O)(jy - 0.5 * p.g[1]);
-            u[2 * N + node] = (O)(jz - 0.5 * p.g[2]);
+    const int t = threadIdx.x;
+    const bool inc = p.eq == LBM_EQ_INCOMPR;
+    const double hg[3] = {0.5 * p.g[0], 0.5 * p.g[1], 0.5 * p.g[2]};
+    for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
+        const int4 hd = groups[g];
+        if (t >= hd.w) continue;
+        const typename Store<DT>::T* src = f + (p.sg0 + g) * (Q * GROUP_LANES) + t;
+        const uint32_t gi = fidx[hd.z + t];
+        NodeFields<O> o;
+        FixMoments fm;
+        PairMoments pm = {};
+        if constexpr (DT == LBM_F64) fm = fix_node_moments(src);
+        else add_node_moments<DT>(src, pm);
+        // the plain FP64 form: FP64 results of the other formats, and nodes whose density lies
+        // outside the ranges of the forms below
+        auto wide = [&]() {
+            double m[4];
+            if constexpr (DT == LBM_F64) {
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                m[0] = fm.nonfinite ? nan : fix_to_double(fm.r);
+                for (int a = 0; a < 3; a++) m[1 + a] = fm.nonfinite ? nan : fix_to_double(fm.j[a]);
+            } else {
+                for (int c = 0; c < 4; c++) m[c] = (double)pm.s[c] + (double)pm.e[c];
+                m[0] += 1.0;
+            }
+            const double half[3] = {0.5 * (gfield_c ? (double)gfield_c[hd.z + t] : p.g[0]), 0.5 * p.g[1], 0.5 * p.g[2]};
+            const NodeFields<double> w = fields_of(m, half, inc);
+            o.rho = (O)w.rho;
+            for (int a = 0; a < 3; a++) o.u[a] = (O)w.u[a];
+        };
+        if constexpr (sizeof(O) == 8) {
+            if constexpr (DT == LBM_F64) {
+                bool ok;
+                const double half[3] = {gfield_c ? 0.5 * gfield_c[hd.z + t] : hg[0], hg[1], hg[2]};
+                o = fields_of(fm, half, inc, ok);
+                if (!ok) wide();
+            } else {
+                wide();
+            }
         } else {
-            u[node] = (O)((jx - 0.5 * Fx) / r);
-            u[N + node] = (O)((jy - 0.5 * p.g[1]) / r);
-            u[2 * N + node] = (O)((jz - 0.5 * p.g[2]) / r);
+            dfl r, j[3], half[3];
+            if constexpr (DT == LBM_F64) half[0] = gfield_c ? df_from_double(gfield_c[hd.z + t]) : p.dfc.Fx;
+            else half[0] = gfield_c ? df_make(gfield_c[hd.z + t], 0.f) : p.dfc.Fx;
+            half[0] = df_scale2(half[0], 0.5f);
+            half[1] = df_scale2(p.dfc.Fy, 0.5f);
+            half[2] = df_scale2(p.dfc.Fz, 0.5f);
+            bool ok;
+            if constexpr (DT == LBM_F64) {
+                r = df_from_fix(fm.r);
+                for (int a = 0; a < 3; a++) j[a] = df_from_fix(fm.j[a]);
+                o = fields_of(r, j, half, inc, ok);
+                ok = ok && !fm.nonfinite;
+            } else {
+                r = df_add_dom(df_make(1.0f, 0.0f), df_make(pm.s[0], pm.e[0]));
+                for (int a = 0; a < 3; a++) j[a] = df_make(pm.s[1 + a], pm.e[1 + a]);
+                o = fields_of(r, j, half, inc, ok);
+                ok = ok && fabsf(pm.s[0]) <= 1.0f;   // 1 dominates
+            }
+            if (!ok) wide();
         }
+        const uint32_t tile = non_empty[gi >> 6];
+        const int s = (int)(gi & 63u);
+        const uint32_t row = tile / (uint32_t)Tx;
+        const int x = TILE * (int)(tile - row * (uint32_t)Tx) + (s & 3);
+        const int y = TILE * (int)(row % (uint32_t)Ty) + ((s >> 2) & 3);
+        const int z = TILE * (int)(row / (uint32_t)Ty) + (s >> 4);
+        const int64_t node = x + (int64_t)nx * (y + (int64_t)ny * z);
+        rho[node] = o.rho;
+        for (int a = 0; a < 3; a++) u[a * N + node] = o.u[a];
     }
 }
 
-template <typename O>
-static void macro_dispatch(lbm_ctx* c, O* rho, O* u) {
-    const OwnTiles o = own_tiles(c);
-    const unsigned g = grid_for(o.n * SLOTS, 256);
-#define LBM_MACRO(DT, TT)                                                                                 \
-    k_macro<DT, O><<<g, 256, 0, c->stream>>>((const TT*)o.f, o.smask, o.tlane, o.non_empty, o.gfield, o.n, c->nx, c->ny, \
-                                             c->nz, c->Tx, c->Ty, c->p, rho, u)
-    if (c->dtype == LBM_F64) LBM_MACRO(LBM_F64, double);
-    else if (c->dtype == LBM_F32) LBM_MACRO(LBM_F32, float);
-    else LBM_MACRO(LBM_F16S, __half);
-#undef LBM_MACRO
+template <int DT, typename O> static void macro_dt(lbm_ctx* c, void* rho, void* u) {
+    const unsigned g = (unsigned)std::min<int64_t>(c->n_groups, 152 * 32);
+    k_macro<DT, O><<<g, MOM_THREADS, 0, c->stream>>>(static_cast<const typename Store<DT>::T*>(c->f[c->cur]), c->groups,
+                                                     c->fidx, c->non_empty, force_c<DT>(c), c->n_groups, c->nx, c->ny,
+                                                     c->nz, c->Tx, c->Ty, c->p, static_cast<O*>(rho),
+                                                     static_cast<O*>(u));
+}
+
+template <int DT> static void macro_out(lbm_ctx* c, void* rho, void* u, int out_f64) {
+    if (out_f64) macro_dt<DT, double>(c, rho, u);
+    else macro_dt<DT, float>(c, rho, u);
 }
 
 cudaError_t launch_macroscopic(lbm_ctx* c, void* rho, void* u, int out_f64) {
-    if (c->own_k1 <= c->own_k0) return cudaSuccess;
-    if (out_f64) macro_dispatch<double>(c, (double*)rho, (double*)u);
-    else macro_dispatch<float>(c, (float*)rho, (float*)u);
+    if (c->n_groups == 0) return cudaSuccess;
+    if (c->dtype == LBM_F64) macro_out<LBM_F64>(c, rho, u, out_f64);
+    else if (c->dtype == LBM_F32) macro_out<LBM_F32>(c, rho, u, out_f64);
+    else macro_out<LBM_F16S>(c, rho, u, out_f64);
     return cudaGetLastError();
 }
 

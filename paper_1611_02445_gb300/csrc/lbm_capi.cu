@@ -204,10 +204,17 @@ void set_mrt_constants(lbm_ctx* c) {
                               r[3], snu, r[3], snu, snu, snu, r[4], r[4], r[4]};
     for (int k = 0; k < lbm::Q; k++) {
         const double n = (double)lbm::mrt_norm(k);
-        c->p.mrt_a[k] = (1.0 - s[k]) / n;
-        c->p.mrt_b[k] = (1.0 - 0.5 * s[k]) / n;
-        c->p.mrt_a_f[k] = (float)c->p.mrt_a[k];
+        // factors of mrt_relax: its n1 is (e + 11 rho) / 19; the Guo moments are multiples of
+        // u.F (e, eps), F (q), 3 u_x F_x - u.F (p_xx, pi_xx) and u_y F_y - u_z F_z (p_ww, pi_ww)
+        const double fs = k == 1 ? 19.0 : 1.0;
+        const double fb = k == 1 ? 38.0 : k == 2 ? -11.0 : k == 4 || k == 6 || k == 8 ? -2.0 / 3.0
+                        : k == 9 || k == 11 ? 2.0 : k == 10 || k == 12 ? -1.0 : 1.0;
+        c->p.mrt_s[k] = fs * s[k] / n;
+        c->p.mrt_b[k] = fb * (1.0 - 0.5 * s[k]) / n;
+        c->p.mrt_s_f[k] = (float)c->p.mrt_s[k];
         c->p.mrt_b_f[k] = (float)c->p.mrt_b[k];
+        c->p.mrt_pa_f[k] = (float)((1.0 - s[k]) / n);
+        c->p.mrt_pb_f[k] = (float)((1.0 - 0.5 * s[k]) / n);
     }
 }
 

@@ -208,11 +208,12 @@ LBM_DF_HD int64_t fix_from_double(double d) {
 // pipe. Any other input (negative, below 2^-6, 16 or more, zero, not finite) sets `bad`
 // and returns an unspecified value; the caller then converts another way. Where this one
 // is valid the value is exact, so fix_from_double and fix_from_double_cvt give the same.
-LBM_DF_HD int64_t fix_from_double_fast(double d, bool& bad) {
+// top: the largest shift taken; 6 narrows the range to 2^-6 <= d < 2.
+LBM_DF_HD int64_t fix_from_double_fast(double d, bool& bad, uint32_t top = 9u) {
     const uint64_t b = bits_of(d);
     const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
     const uint32_t s = (hi >> 20) - 1017u;   // the sign bit makes s large for negative d
-    bad |= s > 9u;
+    bad |= s > top;
     const uint32_t mh = (hi & 0x000fffffu) | 0x00100000u;
 #if defined(__CUDA_ARCH__)
     const uint32_t rh = __funnelshift_l(lo, mh, s);

@@ -157,11 +157,14 @@ struct StepParams {
     // FP32 copies for the 4-byte formats (an FP64 -> FP32 conversion runs on the FP64 pipe)
     float omega_f, beta_f, g_f[3], u_in_f[3], rho_out_f, rho_out_m1_f;
     // collision model (lbm_set_model): equilibrium (LBM_EQ_*) and collision (LBM_COLL_*);
-    // for MRT, moment k relaxes as m*_k = m^eq_k + (1 - s_k)(m_k - m^eq_k) + (1 - s_k/2) mG_k,
-    // kept as mrt_a[k] = (1 - s_k) / |M_k|^2 and mrt_b[k] = (1 - s_k/2) / |M_k|^2
+    // for MRT, moment k relaxes as m*_k = m_k - s_k (m_k - m^eq_k) + (1 - s_k/2) mG_k. mrt_s and
+    // mrt_b: s_k / |M_k|^2 and (1 - s_k/2) / |M_k|^2 times the factors of mrt_relax's moments.
+    // FP16 storage takes the products written out (relax_products) with (1 - s_k) / |M_k|^2 and
+    // (1 - s_k/2) / |M_k|^2.
     int eq, coll;
-    double mrt_a[Q], mrt_b[Q];
-    float mrt_a_f[Q], mrt_b_f[Q];
+    double mrt_s[Q], mrt_b[Q];
+    float mrt_s_f[Q], mrt_b_f[Q];
+    float mrt_pa_f[Q], mrt_pb_f[Q];
     // moving wall (lbm_set_lid): 6 w_i (c_i . u_lid) for the directions whose links cross
     // the lid face from a node on it, 0 for the others
     double lid_c[Q];

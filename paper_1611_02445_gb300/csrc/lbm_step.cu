@@ -323,15 +323,15 @@ __device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int d
     if constexpr (MODE != STEP_FULL) {
         // calibration kernels: no collision, the gathered values are stored as they are
     } else if constexpr (GEN) {
-        // incompressible equilibrium or MRT; for FP64 storage the incompressible LBGK of a
-        // fluid node takes the hybrid collision as well
+        // incompressible equilibrium or MRT; for FP64 storage a fluid node takes its moments
+        // in fixed point, with the hybrid collision for the incompressible LBGK
         if constexpr (DT == LBM_F64 && !VAR) {
             if (type == LBM_FLUID && p.coll == LBM_COLL_BGK && p.eq == LBM_EQ_INCOMPR)
                 collide_df<false, true>(v, (double)Fx, p.dfc, !has_gf);
-            else
-                collide_model<R, false>(v, type, p, Fx, Fy, Fz);
+            else if (type != LBM_FLUID || p.coll != LBM_COLL_MRT || !collide_mrt_fix(v, p, (double)Fx))
+                collide_model<R, false, false>(v, type, p, Fx, Fy, Fz);
         } else {
-            collide_model<R, Store<DT>::SHIFT>(v, type, p, Fx, Fy, Fz);
+            collide_model<R, Store<DT>::SHIFT, DT == LBM_F16S>(v, type, p, Fx, Fy, Fz);
         }
     } else if constexpr (DT == LBM_F64 && !VAR) {
         // FP64 storage: double-float collision for fluid nodes (and Zou-He boundary nodes

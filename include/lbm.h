@@ -225,9 +225,9 @@ lbm_status lbm_set_f(lbm_ctx* ctx, const double* f_dense);
  *             Device pointer if dL_dg_on_device, else host. May be NULL.
  *   dL_dtau   host, receives dL/dtau. May be NULL.
  * Gradients accumulate in FP64; the adjoint arithmetic runs in the storage's arithmetic
- * precision (FP64 for LBM_F64, FP32 otherwise). Device memory: (ceil(T/ckpt_every) +
- * min(ckpt_every, T)) population copies plus two adjoint copies; if it cannot be
- * allocated the call returns LBM_ENOMEM before any work and the state is unchanged.
+ * precision (FP64 for LBM_F64, FP32 otherwise). Device memory, as one allocation released
+ * before the call returns: (ceil(T/ckpt_every) - 1 + min(ckpt_every, T)) population copies
+ * plus two adjoint copies; if it cannot be allocated the call returns LBM_ENOMEM before any work and the state is unchanged.
  * LBM_EUNSUPPORTED for a context of format LBM_F16S_SR (its recompute would not
  * reproduce the forward's random rounding without storing the counter per segment),
  * with a model other than quasi-compressible LBGK, a moving wall or Zou-He boundaries. */

@@ -265,6 +265,9 @@ namespace lbm {
 cudaError_t dmalloc(void** p, size_t bytes);
 void dfree(void* p);
 
+// 32-bit gather indices when every element index of a copy fits.
+inline bool idx32(const lbm_ctx* c) { return c->p.n_padded * (int64_t)Q < (int64_t(1) << 31); }
+
 // Launchers (defined in lbm_tiles.cu / lbm_step.cu); all queue work on ctx->stream and
 // return cudaGetLastError() of the launch.
 cudaError_t launch_tile_flags(const uint8_t* nt, int nx, int ny, int nz, int Tx, int Ty, int Tz,

@@ -33,6 +33,7 @@
 #include <cstddef>
 #include <type_traits>
 
+#include "lbm_async.cuh"
 #include "lbm_collide.cuh"
 #include "lbm_internal.cuh"
 #include "lbm_store.cuh"
@@ -72,29 +73,6 @@ static_assert(StepCfg<LBM_F32>::THREADS == GROUP_MAX_NODES && StepCfg<LBM_F64>::
 constexpr int HDR_SLOTS = 4;
 constexpr int META_SLOTS = 3;
 constexpr int REC_SLOTS = 2;
-
-// ---------------------------------------------------------------------------- cp.async
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async8_sa(unsigned sa, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4_sa(unsigned sa, const void* gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // ------------------------------------------------------------------- checked build
 // With LBM_CHECKED every index the step takes from its tables is tested before use; a
@@ -488,9 +466,6 @@ static int step_grid(int64_t n_groups, bool with_gf) {
     }
     return (int)std::max<int64_t>(1, std::min<int64_t>(n_groups, (int64_t)ps * n_sm));
 }
-
-// 32-bit gather indices when every element index of a copy fits (issue_gather).
-static bool idx32(const lbm_ctx* c) { return c->p.n_padded * (int64_t)Q < (int64_t(1) << 31); }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool I32>
 static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B) {

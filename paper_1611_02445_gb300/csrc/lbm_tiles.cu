@@ -235,12 +235,27 @@ cudaError_t launch_node_words(lbm_ctx* c) {
 
 // ----------------------------------------------------------------------------------
 // Equilibrium initial state f = f^eq(rho0, u0) (Eq. 3) of every non-solid node, in both
-// copies.
+// copies. The 19 values are the same everywhere: a CTA forms them once in FP64 and keeps them
+// stored in shared memory. (Formed per node they were all FP64-pipe time: 364 us on a 128^3
+// pack in FP32.)
 template <int DT>
 __global__ void k_init(typename Store<DT>::T* __restrict__ f0, typename Store<DT>::T* __restrict__ f1,
                        const uint64_t* __restrict__ smask, const int32_t* __restrict__ tlane, int64_t n_tiles,
                        double rho0, double ux, double uy, double uz, int eq) {
     using T = typename Store<DT>::T;
+    __shared__ T value[Q];
+    if (threadIdx.x == 0) {
+        const double uu = ux * ux + uy * uy + uz * uz;
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            const double cu = cx(i) * ux + cy(i) * uy + cz(i) * uz;
+            // Eq. 3, or Eq. 4 for the incompressible model
+            const double fe = eq == LBM_EQ_INCOMPR ? wgt(i) * (rho0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu)
+                                                   : wgt(i) * rho0 * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
+            value[i] = from_f64<DT>(fe, i);
+        }
+    }
+    __syncthreads();
     const int64_t n = n_tiles * SLOTS;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -249,14 +264,9 @@ __global__ void k_init(typename Store<DT>::T* __restrict__ f0, typename Store<DT
         const uint64_t sm = smask[k];
         if ((sm >> s) & 1) continue;   // solid slots have no storage
         const uint32_t P = node_lane((uint32_t)tlane[k], sm, s);
-        const double uu = ux * ux + uy * uy + uz * uz;
 #pragma unroll
         for (int i = 0; i < Q; i++) {
-            const double cu = cx(i) * ux + cy(i) * uy + cz(i) * uz;
-            // Eq. 3, or Eq. 4 for the incompressible model
-            const double fe = eq == LBM_EQ_INCOMPR ? wgt(i) * (rho0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu)
-                                                   : wgt(i) * rho0 * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-            const T v = from_f64<DT>(fe, i);
+            const T v = value[i];
             f0[data_index(P, i)] = v;
             f1[data_index(P, i)] = v;
         }
@@ -333,7 +343,7 @@ cudaError_t launch_node_records(lbm_ctx* c) {
 }
 
 cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]) {
-    const unsigned g = grid_for(c->n_tiles * SLOTS, 256);
+    const unsigned g = std::min(grid_for(c->n_tiles * SLOTS, 256), 152u * 8u);
     switch (c->dtype) {
         case LBM_F64:
             k_init<LBM_F64><<<g, 256, 0, c->stream>>>((double*)c->f[0], (double*)c->f[1], c->smask, c->tlane,

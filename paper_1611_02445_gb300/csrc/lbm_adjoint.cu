@@ -274,11 +274,12 @@ template <int DT> struct AdjSmem {
 
 template <int DT, bool XF, bool I32>
 __global__ void __launch_bounds__(ADJ_THREADS, adj_ctas<DT>())
-k_adjoint(const typename Store<DT>::T* __restrict__ st, const typename Store<DT>::T* __restrict__ sT,
-          const Arith<DT>* __restrict__ mu_in, Arith<DT>* __restrict__ mu_out, NodeTables nt,
+k_adjoint(const typename Store<DT>::T* st, const typename Store<DT>::T* sT, const Arith<DT>* mu_in,
+          Arith<DT>* mu_out, NodeTables nt,   // not __restrict__: the launch before may still write them
+
           const int64_t* __restrict__ nrec, const uint32_t* __restrict__ fword, const uint4* __restrict__ frank,
-          const Arith<DT>* __restrict__ gfield_c, StepParams p, const double* __restrict__ sums,
-          double* __restrict__ gbar, double* __restrict__ tau_part) {
+          const Arith<DT>* __restrict__ gfield_c, StepParams p, const double* __restrict__ sums, double* gbar,
+          double* tau_part) {
     using R = Arith<DT>;
     using IX = typename std::conditional<I32, int32_t, int64_t>::type;
     constexpr int CH = NBR_STRIDE / 2;   // 16-byte chunks of a tile's records
@@ -303,7 +304,7 @@ k_adjoint(const typename Store<DT>::T* __restrict__ st, const typename Store<DT>
             }
         }
     };
-    const int64_t g0 = blockIdx.x;
+    const int64_t g0 = G - 1 - blockIdx.x;   // as in the step: the CTAs with one group more come last
     issue_header(g0, 0);
     issue_header(g0 + G, 1);
     cp_async_commit();
@@ -311,6 +312,7 @@ k_adjoint(const typename Store<DT>::T* __restrict__ st, const typename Store<DT>
     __syncthreads();
     issue_meta(g0, 0);
     cp_async_commit();
+    grid_wait();   // the tables are constant; from here on the launch before is complete
     R tau1 = R(0), tau2 = R(0), err1 = R(0), err2 = R(0);
     int it = 0;
     for (int64_t g = g0; g < nt.n_groups; g += G, it++) {
@@ -351,7 +353,7 @@ k_adjoint(const typename Store<DT>::T* __restrict__ st, const typename Store<DT>
         const R Fx = gfield_c ? sm.gf[slot][t] : par<R>(p.g[0], p.g_f[0]);
         double gb = 0.0;
         if (!sT) {
-            gb = gbar[n];
+            gb = __ldcg(gbar + n);
         } else {
             const bool plane = nt.x_of(n) == nt.plane_x;
             double r = 1.0, ux = 0.0;
@@ -383,7 +385,7 @@ k_adjoint(const typename Store<DT>::T* __restrict__ st, const typename Store<DT>
     }
     cp_async_wait<0>();
     const double total = block_sum(((double)tau1 + (double)err1) + 0.5 * ((double)tau2 + (double)err2), sm.sum);
-    if (t == 0) tau_part[g0] += total;   // times omega^2: applied to the sum
+    if (t == 0) tau_part[g0] = __ldcg(tau_part + g0) + total;   // times omega^2: applied to the sum
 }
 
 // Per-node gradient in group order -> dense array (zeroed by the caller).
@@ -425,18 +427,14 @@ template <int DT> int64_t adj_grid(const lbm_ctx* c) {
 
 template <int DT, bool XF>
 cudaError_t launch_reverse(lbm_ctx* c, const void* st, const void* sT, const Arith<DT>* mu_in, Arith<DT>* mu_out,
-                           const NodeTables& nt, const double* sums, double* gbar, double* taup) {
+                           const NodeTables& nt, const double* sums, double* gbar, double* taup, bool chained) {
     using TT = typename Store<DT>::T;
     const Arith<DT>* gf = c->gfield ? static_cast<const Arith<DT>*>(c->gfield_c) : nullptr;
     const TT *a = static_cast<const TT*>(st), *b = static_cast<const TT*>(sT);
     const unsigned grid = (unsigned)adj_grid<DT>(c);
-    if (idx32(c))
-        k_adjoint<DT, XF, true><<<grid, ADJ_THREADS, 0, c->stream>>>(a, b, mu_in, mu_out, nt, c->nrec, c->fword, c->frank,
-                                                                    gf, c->p, sums, gbar, taup);
-    else
-        k_adjoint<DT, XF, false><<<grid, ADJ_THREADS, 0, c->stream>>>(a, b, mu_in, mu_out, nt, c->nrec, c->fword, c->frank,
-                                                                     gf, c->p, sums, gbar, taup);
-    return cudaGetLastError();
+    return launch_chained(idx32(c) ? k_adjoint<DT, XF, true> : k_adjoint<DT, XF, false>, grid, (unsigned)ADJ_THREADS, 0,
+                          c->stream, chained, a, b, mu_in, mu_out, nt, c->nrec, c->fword, c->frank, gf, c->p, sums, gbar,
+                          taup);
 }
 
 template <int DT>
@@ -482,7 +480,7 @@ cudaError_t run_adjoint(lbm_ctx* c, int T, int K, int plane_x, double* loss, dou
     const auto first_of = [&](int sgi) -> const void* { return sgi == 0 ? s0 : ckp + copy * (sgi - 1); };
     if (!grads) {
         for (int t = 0; t < T; t++) {
-            if ((e = launch_step(c, c->f[c->cur], c->f[1 - c->cur])) != cudaSuccess) return e;
+            if ((e = launch_step(c, c->f[c->cur], c->f[1 - c->cur], t > 0)) != cudaSuccess) return e;
             c->cur ^= 1;
         }
     } else {
@@ -494,7 +492,7 @@ cudaError_t run_adjoint(lbm_ctx* c, int T, int K, int plane_x, double* loss, dou
             else if ((t + 1) % K == 0) to = ckp + copy * ((t + 1) / K - 1);
             else if (t + 1 > t_last) to = sb + copy * (t + 1 - t_last);
             else to = from == other ? static_cast<void*>(sb) : other;
-            if ((e = launch_step(c, from, to)) != cudaSuccess) return e;
+            if ((e = launch_step(c, from, to, t > 0)) != cudaSuccess) return e;
             from = to;
         }
         c->cur ^= 1;
@@ -528,16 +526,16 @@ cudaError_t run_adjoint(lbm_ctx* c, int T, int K, int plane_x, double* loss, dou
     const auto reverse = [&](const void* st, const void* seed) {
         mcur ^= 1;
         return xf ? launch_reverse<DT, true>(c, st, seed, mu[1 - mcur], mu[mcur], nt, ws.at<double>(sums),
-                                             ws.at<double>(gbar), ws.at<double>(taup))
+                                             ws.at<double>(gbar), ws.at<double>(taup), !seed)
                   : launch_reverse<DT, false>(c, st, seed, mu[1 - mcur], mu[mcur], nt, ws.at<double>(sums),
-                                              ws.at<double>(gbar), ws.at<double>(taup));
+                                              ws.at<double>(gbar), ws.at<double>(taup), !seed);
     };
     for (int sgi = n_ck - 1; sgi >= 0; sgi--) {
         const int t0 = sgi * K, t1 = std::min(T, t0 + K);
         const auto state = [&](int t) -> const void* { return t == t0 ? first_of(sgi) : sb + copy * (t - t0); };
         if (sgi != n_ck - 1)
             for (int t = t0 + 1; t < t1; t++)
-                if ((e = launch_step(c, state(t - 1), sb + copy * (t - t0))) != cudaSuccess) return e;
+                if ((e = launch_step(c, state(t - 1), sb + copy * (t - t0), true)) != cudaSuccess) return e;
         for (int t = t1 - 1; t >= t0; t--)
             if ((e = reverse(state(t), t == T - 1 ? sT : nullptr)) != cudaSuccess) return e;
     }

@@ -111,7 +111,7 @@ cudaError_t build_graph(lbm_ctx* c, int start) {
     if (e == cudaSuccess) {
         int cur = start;
         for (int k = 0; k < lbm::GRAPH_STEPS && e == cudaSuccess; k++) {
-            e = lbm::launch_step(c, c->f[cur], c->f[1 - cur]);
+            e = lbm::launch_step(c, c->f[cur], c->f[1 - cur], k > 0);
             cur ^= 1;
         }
         cudaError_t e2 = cudaStreamEndCapture(cap, &g);
@@ -781,7 +781,7 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
         }
     }
     for (; k < n; k++) {
-        LBM_CUDA(c, lbm::launch_step(c, c->f[c->cur], c->f[1 - c->cur]));
+        LBM_CUDA(c, lbm::launch_step(c, c->f[c->cur], c->f[1 - c->cur], k > 0));
         c->cur ^= 1;
     }
     return read_check(c);
@@ -793,7 +793,7 @@ lbm_status lbm_step_kernel(lbm_ctx* c, int kind, int n) {
     if (kind < LBM_KERNEL_FULL || kind > LBM_KERNEL_RW) return fail(c, LBM_EINVAL, "unknown kernel kind");
     if (!c->state_set || !c->params_set) return fail(c, LBM_ESTATE, "set parameters and a state before stepping");
     for (int k = 0; k < n; k++) {
-        LBM_CUDA(c, lbm::launch_step_kind(c, kind, c->f[c->cur], c->f[1 - c->cur]));
+        LBM_CUDA(c, lbm::launch_step_kind(c, kind, c->f[c->cur], c->f[1 - c->cur], k > 0));
         c->cur ^= 1;
     }
     return read_check(c);

@@ -280,8 +280,10 @@ cudaError_t launch_node_words(lbm_ctx* c);
 cudaError_t launch_lane_lists(lbm_ctx* c, const int64_t* lane0, const uint8_t* lt);
 cudaError_t launch_node_records(lbm_ctx* c);
 cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]);
-cudaError_t launch_step(lbm_ctx* c, const void* A, void* B);
-cudaError_t launch_step_kind(lbm_ctx* c, int kind, const void* A, void* B);
+// chained: the launch directly before on the stream is a step or adjoint launch of the same
+// call (lbm_async.cuh).
+cudaError_t launch_step(lbm_ctx* c, const void* A, void* B, bool chained);
+cudaError_t launch_step_kind(lbm_ctx* c, int kind, const void* A, void* B, bool chained);
 cudaError_t prepare_step(lbm_ctx* c);
 cudaError_t launch_reduce(lbm_ctx* c, double* d_out);
 cudaError_t launch_macroscopic(lbm_ctx* c, void* rho, void* u, int out_f64);

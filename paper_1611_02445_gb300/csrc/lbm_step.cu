@@ -363,17 +363,11 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
        uint32_t* __restrict__ seed_out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StepSmem<DT>& sm = *reinterpret_cast<StepSmem<DT>*>(smem_raw);
-    const int64_t G = gridDim.x;
-    const int64_t g0 = blockIdx.x;
-    uint32_t key = 0;
-    if (DT == LBM_F16S && VAR) {
-        // step counter of the rounding hash: read from this launch's copy, advanced into
-        // the other copy's, which no thread of this launch reads
-        const uint32_t t = *seed_in;
-        if (blockIdx.x == 0 && threadIdx.x == 0) *seed_out = t + 1u;
-        key = fmix32(t * 0x9e3779b9u + 0x7f4a7c15u);
-    }
-    if (g0 >= n_groups) return;
+    const int64_t G = gridDim.x;   // at most n_groups
+    // The CTAs with one group more than the others are the last ones: a chained launch's CTAs
+    // start in index order on the places that become free, so those with fewer groups follow
+    // each other on the same SMs and so do the others, as the first launch spread them.
+    const int64_t g0 = G - 1 - blockIdx.x;
     const bool has_gf = gfield_c != nullptr;
     // prologue: headers of groups 0..2, meta of groups 0..1, gathers of group 0
     issue_hdr(&sm.hdr[0], g0, n_groups, groups);
@@ -390,6 +384,15 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
     cp_async_commit();
     cp_async_wait<1>();
     __syncthreads();
+    grid_wait();   // the tables above are constant; from here on the launch before is complete
+    uint32_t key = 0;
+    if (DT == LBM_F16S && VAR) {
+        // step counter of the rounding hash: read from this launch's copy, advanced into
+        // the other copy's, which no thread of this launch reads
+        const uint32_t t = __ldcg(seed_in);
+        if (blockIdx.x == 0 && threadIdx.x == 0) *seed_out = t + 1u;
+        key = fmix32(t * 0x9e3779b9u + 0x7f4a7c15u);
+    }
     issue_gather<DT, MODE, I32>(sm, 0, 0, 0, group_header<DT>(sm.hdr[0], p), p.sg0 + g0, A, p, 0u);
     cp_async_commit();
     constexpr int NS = StepCfg<DT>::SLOTS;
@@ -468,7 +471,7 @@ static int step_grid(int64_t n_groups, bool with_gf) {
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool I32>
-static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B) {
+static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B, bool chained) {
     using T = typename Store<DT>::T;
     const bool with_gf = c->gfield != nullptr;
     const int grid = step_grid<DT, VAR, MODE, GEN, XF, I32>(c->n_groups, with_gf);
@@ -476,16 +479,15 @@ static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B) {
     const int from = A == c->f[0] ? 0 : 1;
     const uint32_t* seed_in = c->seed ? c->seed + from : nullptr;
     uint32_t* seed_out = c->seed ? c->seed + (1 - from) : nullptr;
-    k_step<DT, VAR, MODE, GEN, XF, I32><<<grid, StepCfg<DT>::THREADS, step_smem<DT>(with_gf), c->stream>>>(
-        (const T*)A, (T*)B, c->groups, c->nrec, c->fword, c->frank, c->gfield ? c->gfield_c : nullptr, c->n_groups, c->p,
-        seed_in, seed_out);
-    return cudaGetLastError();
+    return launch_chained(k_step<DT, VAR, MODE, GEN, XF, I32>, (unsigned)grid, (unsigned)StepCfg<DT>::THREADS,
+                          step_smem<DT>(with_gf), c->stream, chained, (const T*)A, (T*)B, c->groups, c->nrec, c->fword,
+                          c->frank, c->gfield ? c->gfield_c : nullptr, c->n_groups, c->p, seed_in, seed_out);
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF>
-static cudaError_t launch_step_xf(lbm_ctx* c, const void* A, void* B) {
-    return idx32(c) ? launch_step_ix<DT, VAR, MODE, GEN, XF, true>(c, A, B)
-                    : launch_step_ix<DT, VAR, MODE, GEN, XF, false>(c, A, B);
+static cudaError_t launch_step_xf(lbm_ctx* c, const void* A, void* B, bool chained) {
+    return idx32(c) ? launch_step_ix<DT, VAR, MODE, GEN, XF, true>(c, A, B, chained)
+                    : launch_step_ix<DT, VAR, MODE, GEN, XF, false>(c, A, B, chained);
 }
 
 // The instantiations with the hybrid FP64 collision (FP64 storage, hybrid arithmetic,
@@ -497,11 +499,11 @@ constexpr bool has_xf_form() {
 static bool force_along_x(const lbm_ctx* c) { return c->p.g[1] == 0.0 && c->p.g[2] == 0.0; }
 
 template <int DT, bool VAR, int MODE, bool GEN>
-static cudaError_t launch_step_dt(lbm_ctx* c, const void* A, void* B) {
+static cudaError_t launch_step_dt(lbm_ctx* c, const void* A, void* B, bool chained) {
     if constexpr (has_xf_form<DT, VAR, MODE, GEN>()) {
-        if (force_along_x(c)) return launch_step_xf<DT, VAR, MODE, GEN, true>(c, A, B);
+        if (force_along_x(c)) return launch_step_xf<DT, VAR, MODE, GEN, true>(c, A, B, chained);
     }
-    return launch_step_xf<DT, VAR, MODE, GEN, false>(c, A, B);
+    return launch_step_xf<DT, VAR, MODE, GEN, false>(c, A, B, chained);
 }
 
 template <int DT, bool VAR, bool GEN, bool I32>
@@ -518,26 +520,28 @@ static void prepare_dt(lbm_ctx* c) {
 }
 
 template <int MODE, bool GEN>
-static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B) {
+static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B, bool chained) {
     switch (c->dtype) {
         case LBM_F64:
-            return c->native64 ? launch_step_dt<LBM_F64, true, MODE, GEN>(c, A, B)
-                               : launch_step_dt<LBM_F64, false, MODE, GEN>(c, A, B);
-        case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN>(c, A, B);
+            return c->native64 ? launch_step_dt<LBM_F64, true, MODE, GEN>(c, A, B, chained)
+                               : launch_step_dt<LBM_F64, false, MODE, GEN>(c, A, B, chained);
+        case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN>(c, A, B, chained);
         default:
-            return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN>(c, A, B)
-                         : launch_step_dt<LBM_F16S, false, MODE, GEN>(c, A, B);
+            return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN>(c, A, B, chained)
+                         : launch_step_dt<LBM_F16S, false, MODE, GEN>(c, A, B, chained);
     }
 }
 
 // The calibration kernels have no collision, so only the fused step has model variants.
 template <int MODE>
-static cudaError_t launch_step_mode(lbm_ctx* c, const void* A, void* B) {
-    if (MODE == STEP_FULL && c->gen) return launch_step_model<STEP_FULL, true>(c, A, B);
-    return launch_step_model<MODE, false>(c, A, B);
+static cudaError_t launch_step_mode(lbm_ctx* c, const void* A, void* B, bool chained) {
+    if (MODE == STEP_FULL && c->gen) return launch_step_model<STEP_FULL, true>(c, A, B, chained);
+    return launch_step_model<MODE, false>(c, A, B, chained);
 }
 
-cudaError_t launch_step(lbm_ctx* c, const void* A, void* B) { return launch_step_kind(c, STEP_FULL, A, B); }
+cudaError_t launch_step(lbm_ctx* c, const void* A, void* B, bool chained) {
+    return launch_step_kind(c, STEP_FULL, A, B, chained);
+}
 
 // One-time kernel attributes and occupancy query of the fused step, done outside any
 // stream capture.
@@ -561,12 +565,12 @@ cudaError_t prepare_step(lbm_ctx* c) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_kind(lbm_ctx* c, int kind, const void* A, void* B) {
+cudaError_t launch_step_kind(lbm_ctx* c, int kind, const void* A, void* B, bool chained) {
     if (c->n_groups == 0) return cudaSuccess;
     switch (kind) {
-        case STEP_PROPAGATE: return launch_step_mode<STEP_PROPAGATE>(c, A, B);
-        case STEP_RW: return launch_step_mode<STEP_RW>(c, A, B);
-        default: return launch_step_mode<STEP_FULL>(c, A, B);
+        case STEP_PROPAGATE: return launch_step_mode<STEP_PROPAGATE>(c, A, B, chained);
+        case STEP_RW: return launch_step_mode<STEP_RW>(c, A, B, chained);
+        default: return launch_step_mode<STEP_FULL>(c, A, B, chained);
     }
 }
 

@@ -289,6 +289,30 @@ __device__ __forceinline__ void relax_products(float v[Q], const float ve[Q], co
     }
 }
 
+// Equilibrium closure of an inlet or outlet node for the incompressible model in FP64 (Eq. 4):
+// w (rho + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u) with the node's density and u_in, or rho_out and the
+// node's u = j + F/2.
+__device__ __forceinline__ void closure_inc(double v[Q], int type, const StepParams& p, double Fx, double Fy, double Fz) {
+    double r = 0.0, ux = 0.5 * Fx, uy = 0.5 * Fy, uz = 0.5 * Fz;
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        r += v[i];
+        if (cx(i)) ux += cx(i) > 0 ? v[i] : -v[i];
+        if (cy(i)) uy += cy(i) > 0 ? v[i] : -v[i];
+        if (cz(i)) uz += cz(i) > 0 ? v[i] : -v[i];
+    }
+    if (type == LBM_INLET) {
+        ux = p.u_in[0];
+        uy = p.u_in[1];
+        uz = p.u_in[2];
+    } else {
+        r = p.rho_out;
+    }
+    const double uu15 = 1.5 * (ux * ux + uy * uy + uz * uz);
+#pragma unroll
+    for (int i = 0; i < Q; i++) v[i] = feq_model<double>(i, r, 1.0, ux, uy, uz, uu15);
+}
+
 // MRT collision of a fluid node (Eq. 8), in place: v* = v + M^T t with
 //   t_k = ((1 - s_k / 2) G_k - s_k (m_k - m^eq_k)) / |M_k|^2,  m = M v,
 // G the moments of the Guo term w_i (3 (c_i - u).F + 9 (c_i.u)(c_i.F)). The moments of the
@@ -346,34 +370,36 @@ template <typename T> __device__ __forceinline__ MrtMoments<T> mrt_moments(const
 }
 
 // v += M^T t from the moments, J and u. p.mrt_s and p.mrt_b hold the rates with |M_k|^2 and the
-// factors above folded in (StepParams).
-template <typename R>
+// factors above folded in (StepParams). XF: the force has no y or z component.
+template <typename R, bool XF>
 __device__ __forceinline__ void mrt_relax(R v[Q], const MrtMoments<R>& n, const R J[3], const R u[3], const R F[3],
                                           const StepParams& p) {
     const auto ks = [&](int k) { return par<R>(p.mrt_s[k], p.mrt_s_f[k]); };
     const auto kb = [&](int k) { return par<R>(p.mrt_b[k], p.mrt_b_f[k]); };
     const R exx = J[0] * u[0], eyy = J[1] * u[1], ezz = J[2] * u[2], ju = exx + eyy + ezz;
-    const R gxx = u[0] * F[0], gyy = u[1] * F[1], gzz = u[2] * F[2], uF = gxx + gyy + gzz;
-    const R exn = R(3) * exx - ju, gxn = R(3) * gxx - uF, ewn = eyy - ezz, gwn = gyy - gzz;
+    const R gxx = u[0] * F[0], gyy = XF ? R(0) : u[1] * F[1], gzz = XF ? R(0) : u[2] * F[2];
+    const R uF = XF ? gxx : gxx + gyy + gzz;
+    const R exn = R(3) * exx - ju, gxn = XF ? R(2) * gxx : R(3) * gxx - uF, ewn = eyy - ezz, gwn = gyy - gzz;
     const R t1 = kb(1) * uF - ks(1) * (n.n1 - ju);
     const R t2 = kb(2) * uF - ks(2) * (n.n2 + R(5.5) * ju);
     const R t4 = kb(4) * F[0] - ks(4) * (n.nq[0] + R(2.0 / 3.0) * J[0]);
-    const R t6 = kb(6) * F[1] - ks(6) * (n.nq[1] + R(2.0 / 3.0) * J[1]);
-    const R t8 = kb(8) * F[2] - ks(8) * (n.nq[2] + R(2.0 / 3.0) * J[2]);
+    const R q6 = ks(6) * (n.nq[1] + R(2.0 / 3.0) * J[1]), q8 = ks(8) * (n.nq[2] + R(2.0 / 3.0) * J[2]);
+    const R t6 = XF ? -q6 : kb(6) * F[1] - q6, t8 = XF ? -q8 : kb(8) * F[2] - q8;
     const R t9 = kb(9) * gxn - ks(9) * (n.pxx - exn);
     const R t10 = kb(10) * gxn - ks(10) * (n.pixx + R(0.5) * exn);
-    const R t11 = kb(11) * gwn - ks(11) * (n.pww - ewn);
-    const R t12 = kb(12) * gwn - ks(12) * (n.piww + R(0.5) * ewn);
-    const R t13 = kb(13) * (u[0] * F[1] + u[1] * F[0]) - ks(13) * (n.pxy - J[0] * u[1]);
-    const R t14 = kb(14) * (u[1] * F[2] + u[2] * F[1]) - ks(14) * (n.pyz - J[1] * u[2]);
-    const R t15 = kb(15) * (u[0] * F[2] + u[2] * F[0]) - ks(15) * (n.pxz - J[0] * u[2]);
+    const R q11 = ks(11) * (n.pww - ewn), q12 = ks(12) * (n.piww + R(0.5) * ewn);
+    const R t11 = XF ? -q11 : kb(11) * gwn - q11, t12 = XF ? -q12 : kb(12) * gwn - q12;
+    const R q13 = ks(13) * (n.pxy - J[0] * u[1]), q14 = ks(14) * (n.pyz - J[1] * u[2]), q15 = ks(15) * (n.pxz - J[0] * u[2]);
+    const R t13 = kb(13) * (XF ? u[1] * F[0] : u[0] * F[1] + u[1] * F[0]) - q13;
+    const R t14 = XF ? -q14 : kb(14) * (u[1] * F[2] + u[2] * F[1]) - q14;
+    const R t15 = kb(15) * (XF ? u[2] * F[0] : u[0] * F[2] + u[2] * F[0]) - q15;
     const R t16 = ks(16) * n.m[0], t17 = ks(17) * n.m[1], t18 = ks(18) * n.m[2];   // -t_k
     const R t3 = R(0.1) * F[0], t5 = R(0.1) * F[1], t7 = R(0.1) * F[2];            // |M_j|^2 = 10
     // even part of each plane, odd part of each axis
     const R Ba = R(-11) * t1 - R(4) * t2, Bd = R(8) * t1 + t2;
     const R h = t9 - R(2) * t10, k = t11 - R(2) * t12, r = t9 + t10, w = t11 + t12;
     const R Exy = (Bd + r) + w, Exz = (Bd + r) - w, Eyz = Bd - R(2) * r;
-    const R x3 = t3 + t4, y3 = t5 + t6, z3 = t7 + t8;
+    const R x3 = t3 + t4, y3 = XF ? t6 : t5 + t6, z3 = XF ? t8 : t7 + t8;
     const R Xp = x3 - t16, Xm = x3 + t16, Yp = y3 - t17, Ym = y3 + t17, Zp = z3 - t18, Zm = z3 + t18;
     const auto put = [&](int i, int j, R E, R O) {
         v[i] += E + O;
@@ -381,8 +407,8 @@ __device__ __forceinline__ void mrt_relax(R v[Q], const MrtMoments<R>& n, const 
     };
     v[0] += R(12) * t2 - R(30) * t1;
     put(1, 3, Ba + R(2) * h, t3 - R(4) * t4);
-    put(2, 4, (Ba - h) + k, t5 - R(4) * t6);
-    put(5, 6, (Ba - h) - k, t7 - R(4) * t8);
+    put(2, 4, (Ba - h) + k, XF ? R(-4) * t6 : t5 - R(4) * t6);
+    put(5, 6, (Ba - h) - k, XF ? R(-4) * t8 : t7 - R(4) * t8);
     put(7, 9, Exy + t13, Xp + Ym);
     put(8, 10, Exy - t13, Ym - Xp);
     put(11, 14, Exz + t15, Xm + Zp);
@@ -406,19 +432,21 @@ __device__ __forceinline__ void collide_mrt(R v[Q], const StepParams& p, R Fx, R
         J[a] = n.j[a] + R(0.5) * F[a];
         u[a] = J[a] * ir;
     }
-    mrt_relax(v, n, J, u, F, p);
+    mrt_relax<R, false>(v, n, J, u, F, p);
 }
 
 // FP64 storage: the moments exactly, in 64-bit fixed point, each widened to the nearest FP64
 // value with integer instructions; 1/rho in pairs with one FP64 Newton step. FP64 is left with
 // the relaxation and M^T t, about 150 operations a node, and bounds the step (2 lanes per SM).
 // Porous 128^3 (0.73 M nodes): 1.57 ms a step with 19 x 19 products in FP64 (about 900
-// operations), 0.36 ms with the moments of collide_mrt, 0.25 ms so. The velocity after 15 steps
+// operations), 0.36 ms with the moments of collide_mrt, 0.25 ms so, 0.21 ms for a force along x
+// (XF). The velocity after 15 steps
 // is off by 1.8e-13 relative to long double (9.5e-13 with the products).
 // For populations in [2^-6, 2) and a density below 3: no moment then leaves 64 bits (the
 // largest is eps - 3 rho, below 27 of the 32 that fit; the sum of 19 such values is below 38,
 // and one of 32 or more would come out negative). Any other node is left as it is and
 // refused: it takes FP64 throughout.
+template <bool XF>
 __device__ __forceinline__ bool collide_mrt_fix(double v[Q], const StepParams& p, double Fx) {
     int64_t q[Q];
     bool bad = false;
@@ -450,10 +478,10 @@ __device__ __forceinline__ bool collide_mrt_fix(double v[Q], const StepParams& p
     for (int a = 0; a < 3; a++) {
         n.nq[a] = fix_to_double(m.nq[a]);
         n.m[a] = fix_to_double(m.m[a]);
-        J[a] = __fma_rn(0.5, F[a], fix_to_double(m.j[a]));
+        J[a] = XF && a > 0 ? fix_to_double(m.j[a]) : __fma_rn(0.5, F[a], fix_to_double(m.j[a]));
         u[a] = J[a] * ir;
     }
-    mrt_relax(v, n, J, u, F, p);
+    mrt_relax<double, XF>(v, n, J, u, F, p);
     return true;
 }
 

@@ -254,7 +254,7 @@ __device__ __forceinline__ void store_f16_conserving(const float v[Q], __half* _
 // Read this thread's staged values of group g into registers, let `next` issue the
 // gathers of the thread's node in the next group into the same column, then collide
 // and store. A thread without a node in g still calls next.
-template <int DT, bool VAR, int MODE, bool GEN, bool XF, typename Next>
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, typename Next>
 __device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int dslot, const int4 h, int64_t sg,
                                               typename Store<DT>::T* __restrict__ B, const StepParams& p,
                                               bool has_gf, uint32_t key, Next&& next) {
@@ -300,13 +300,21 @@ __device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int d
     }
     if constexpr (MODE != STEP_FULL) {
         // calibration kernels: no collision, the gathered values are stored as they are
+    } else if constexpr (INC) {
+        // FP64 storage, incompressible LBGK: the hybrid collision for fluid nodes (and Zou-He
+        // boundary nodes once completed)
+        int ct = type;
+        if (ct != LBM_FLUID && p.bc == LBM_BC_ZOU_HE) {
+            zou_he<double, false>(v, ct, p);
+            ct = LBM_FLUID;
+        }
+        if (ct == LBM_FLUID) collide_df<XF, true>(v, (double)Fx, p.dfc, !has_gf);
+        else closure_inc(v, ct, p, (double)Fx, (double)Fy, (double)Fz);
     } else if constexpr (GEN) {
-        // incompressible equilibrium or MRT; for FP64 storage a fluid node takes its moments
-        // in fixed point, with the hybrid collision for the incompressible LBGK
+        // incompressible equilibrium or MRT; for FP64 storage MRT takes a fluid node's moments
+        // in fixed point
         if constexpr (DT == LBM_F64 && !VAR) {
-            if (type == LBM_FLUID && p.coll == LBM_COLL_BGK && p.eq == LBM_EQ_INCOMPR)
-                collide_df<false, true>(v, (double)Fx, p.dfc, !has_gf);
-            else if (type != LBM_FLUID || p.coll != LBM_COLL_MRT || !collide_mrt_fix(v, p, (double)Fx))
+            if (type != LBM_FLUID || p.coll != LBM_COLL_MRT || !collide_mrt_fix<XF>(v, p, (double)Fx))
                 collide_model<R, false, false>(v, type, p, Fx, Fy, Fz);
         } else {
             collide_model<R, Store<DT>::SHIFT, DT == LBM_F16S>(v, type, p, Fx, Fy, Fz);
@@ -354,8 +362,10 @@ constexpr int step_ctas() {
 }
 
 // XF: the FP64 hybrid collision's form for a force along x (F_y = F_z = 0; collide_df).
+// INC: its form for the incompressible equilibrium. (Among the models of GEN, at 2 CTAs per SM and
+// without XF, it ran at 14.2 GLUPS on a 190^3 cavity, 15.3 as a kernel of its own at 3.)
 // I32: 32-bit gather indices (issue_gather).
-template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool I32>
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
 __global__ void __launch_bounds__(StepCfg<DT>::THREADS, step_ctas<DT, GEN>())
 k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __restrict__ B,
        const int4* __restrict__ groups, const int64_t* __restrict__ nrec, const uint32_t* __restrict__ fword,
@@ -423,11 +433,11 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
             // the next group's gathers go into the other slot before this group's are awaited
             gather_next(0u);
             cp_async_wait<3>();   // pending: gather(g), header(g + 3G), meta(g + 2G), gather(g + G)
-            compute_store<DT, VAR, MODE, GEN, XF>(sm, it % META_SLOTS, it % NS, h, p.sg0 + g, B, p, has_gf, key,
+            compute_store<DT, VAR, MODE, GEN, XF, INC>(sm, it % META_SLOTS, it % NS, h, p.sg0 + g, B, p, has_gf, key,
                                               [](uint32_t) {});
         } else {
             // one slot: each thread refills its column once it has read it
-            compute_store<DT, VAR, MODE, GEN, XF>(sm, it % META_SLOTS, 0, h, p.sg0 + g, B, p, has_gf, key, gather_next);
+            compute_store<DT, VAR, MODE, GEN, XF, INC>(sm, it % META_SLOTS, 0, h, p.sg0 + g, B, p, has_gf, key, gather_next);
         }
     }
     cp_async_wait<0>();
@@ -446,7 +456,7 @@ static size_t step_smem(bool with_gf) {
 // (cp.async.ca). Left to itself the driver picks the carveout for the highest occupancy:
 // a light kernel (the calibration kinds) would fit a fifth CTA and keep 28 KB of L1
 // instead of 60 KB, and run 25 % slower.
-template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool I32>
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
 static int step_grid(int64_t n_groups, bool with_gf) {
     static int per_sm[2] = {-1, -1}, n_sm = 0;
     int& ps = per_sm[with_gf ? 1 : 0];
@@ -456,85 +466,90 @@ static int step_grid(int64_t n_groups, bool with_gf) {
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        cudaFuncSetAttribute(k_step<DT, VAR, MODE, GEN, XF, I32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_step<DT, VAR, MODE, GEN, XF, INC, I32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(StepSmem<DT>));
         if (smem_sm > 0) {
             const double need = (double)step_ctas<DT, GEN>() * (double)(sizeof(StepSmem<DT>) + (size_t)reserved);
             const int pct = std::min(100, std::max(1, (int)std::ceil(100.0 * need / smem_sm)));
-            cudaFuncSetAttribute(k_step<DT, VAR, MODE, GEN, XF, I32>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+            cudaFuncSetAttribute(k_step<DT, VAR, MODE, GEN, XF, INC, I32>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         }
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_step<DT, VAR, MODE, GEN, XF, I32>, StepCfg<DT>::THREADS,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_step<DT, VAR, MODE, GEN, XF, INC, I32>, StepCfg<DT>::THREADS,
                                                       step_smem<DT>(with_gf));
         ps = std::max(1, std::min(ps, step_ctas<DT, GEN>()));
     }
     return (int)std::max<int64_t>(1, std::min<int64_t>(n_groups, (int64_t)ps * n_sm));
 }
 
-template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool I32>
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
 static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B, bool chained) {
     using T = typename Store<DT>::T;
     const bool with_gf = c->gfield != nullptr;
-    const int grid = step_grid<DT, VAR, MODE, GEN, XF, I32>(c->n_groups, with_gf);
+    const int grid = step_grid<DT, VAR, MODE, GEN, XF, INC, I32>(c->n_groups, with_gf);
     // the copy read decides which counter is read and which is advanced
     const int from = A == c->f[0] ? 0 : 1;
     const uint32_t* seed_in = c->seed ? c->seed + from : nullptr;
     uint32_t* seed_out = c->seed ? c->seed + (1 - from) : nullptr;
-    return launch_chained(k_step<DT, VAR, MODE, GEN, XF, I32>, (unsigned)grid, (unsigned)StepCfg<DT>::THREADS,
+    return launch_chained(k_step<DT, VAR, MODE, GEN, XF, INC, I32>, (unsigned)grid, (unsigned)StepCfg<DT>::THREADS,
                           step_smem<DT>(with_gf), c->stream, chained, (const T*)A, (T*)B, c->groups, c->nrec, c->fword,
                           c->frank, c->gfield ? c->gfield_c : nullptr, c->n_groups, c->p, seed_in, seed_out);
 }
 
-template <int DT, bool VAR, int MODE, bool GEN, bool XF>
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC>
 static cudaError_t launch_step_xf(lbm_ctx* c, const void* A, void* B, bool chained) {
-    return idx32(c) ? launch_step_ix<DT, VAR, MODE, GEN, XF, true>(c, A, B, chained)
-                    : launch_step_ix<DT, VAR, MODE, GEN, XF, false>(c, A, B, chained);
+    return idx32(c) ? launch_step_ix<DT, VAR, MODE, GEN, XF, INC, true>(c, A, B, chained)
+                    : launch_step_ix<DT, VAR, MODE, GEN, XF, INC, false>(c, A, B, chained);
 }
 
-// The instantiations with the hybrid FP64 collision (FP64 storage, hybrid arithmetic,
-// LBGK, fused step) have a form for a force along x, taken when F_y = F_z = 0.
+// The fused steps of FP64 storage with the hybrid collision or fixed-point MRT moments have a
+// form for a force along x, taken when F_y = F_z = 0.
 template <int DT, bool VAR, int MODE, bool GEN>
 constexpr bool has_xf_form() {
-    return DT == LBM_F64 && !VAR && MODE == STEP_FULL && !GEN;
+    return DT == LBM_F64 && !VAR && MODE == STEP_FULL;
 }
 static bool force_along_x(const lbm_ctx* c) { return c->p.g[1] == 0.0 && c->p.g[2] == 0.0; }
+// The model with the hybrid collision's incompressible form.
+static bool hybrid_inc(const lbm_ctx* c) {
+    return c->dtype == LBM_F64 && !c->native64 && c->p.coll == LBM_COLL_BGK && c->p.eq == LBM_EQ_INCOMPR;
+}
 
-template <int DT, bool VAR, int MODE, bool GEN>
+template <int DT, bool VAR, int MODE, bool GEN, bool INC>
 static cudaError_t launch_step_dt(lbm_ctx* c, const void* A, void* B, bool chained) {
     if constexpr (has_xf_form<DT, VAR, MODE, GEN>()) {
-        if (force_along_x(c)) return launch_step_xf<DT, VAR, MODE, GEN, true>(c, A, B, chained);
+        if (force_along_x(c)) return launch_step_xf<DT, VAR, MODE, GEN, true, INC>(c, A, B, chained);
     }
-    return launch_step_xf<DT, VAR, MODE, GEN, false>(c, A, B, chained);
+    return launch_step_xf<DT, VAR, MODE, GEN, false, INC>(c, A, B, chained);
 }
 
-template <int DT, bool VAR, bool GEN, bool I32>
+template <int DT, bool VAR, bool GEN, bool INC, bool I32>
 static void prepare_ix(lbm_ctx* c) {
     if constexpr (has_xf_form<DT, VAR, STEP_FULL, GEN>())
-        step_grid<DT, VAR, STEP_FULL, GEN, true, I32>(1, c->gfield != nullptr);
-    step_grid<DT, VAR, STEP_FULL, GEN, false, I32>(1, c->gfield != nullptr);
+        step_grid<DT, VAR, STEP_FULL, GEN, true, INC, I32>(1, c->gfield != nullptr);
+    step_grid<DT, VAR, STEP_FULL, GEN, false, INC, I32>(1, c->gfield != nullptr);
 }
 
-template <int DT, bool VAR, bool GEN>
+template <int DT, bool VAR, bool GEN, bool INC>
 static void prepare_dt(lbm_ctx* c) {
-    if (idx32(c)) prepare_ix<DT, VAR, GEN, true>(c);
-    else prepare_ix<DT, VAR, GEN, false>(c);
+    if (idx32(c)) prepare_ix<DT, VAR, GEN, INC, true>(c);
+    else prepare_ix<DT, VAR, GEN, INC, false>(c);
 }
 
 template <int MODE, bool GEN>
 static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B, bool chained) {
     switch (c->dtype) {
         case LBM_F64:
-            return c->native64 ? launch_step_dt<LBM_F64, true, MODE, GEN>(c, A, B, chained)
-                               : launch_step_dt<LBM_F64, false, MODE, GEN>(c, A, B, chained);
-        case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN>(c, A, B, chained);
+            return c->native64 ? launch_step_dt<LBM_F64, true, MODE, GEN, false>(c, A, B, chained)
+                               : launch_step_dt<LBM_F64, false, MODE, GEN, false>(c, A, B, chained);
+        case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN, false>(c, A, B, chained);
         default:
-            return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN>(c, A, B, chained)
-                         : launch_step_dt<LBM_F16S, false, MODE, GEN>(c, A, B, chained);
+            return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN, false>(c, A, B, chained)
+                         : launch_step_dt<LBM_F16S, false, MODE, GEN, false>(c, A, B, chained);
     }
 }
 
 // The calibration kernels have no collision, so only the fused step has model variants.
 template <int MODE>
 static cudaError_t launch_step_mode(lbm_ctx* c, const void* A, void* B, bool chained) {
+    if (MODE == STEP_FULL && hybrid_inc(c)) return launch_step_dt<LBM_F64, false, STEP_FULL, false, true>(c, A, B, chained);
     if (MODE == STEP_FULL && c->gen) return launch_step_model<STEP_FULL, true>(c, A, B, chained);
     return launch_step_model<MODE, false>(c, A, B, chained);
 }
@@ -549,18 +564,19 @@ template <bool GEN>
 static void prepare_model(lbm_ctx* c) {
     switch (c->dtype) {
         case LBM_F64:
-            if (c->native64) prepare_dt<LBM_F64, true, GEN>(c);
-            else prepare_dt<LBM_F64, false, GEN>(c);
+            if (c->native64) prepare_dt<LBM_F64, true, GEN, false>(c);
+            else prepare_dt<LBM_F64, false, GEN, false>(c);
             break;
-        case LBM_F32: prepare_dt<LBM_F32, false, GEN>(c); break;
+        case LBM_F32: prepare_dt<LBM_F32, false, GEN, false>(c); break;
         default:
-            if (c->sr) prepare_dt<LBM_F16S, true, GEN>(c);
-            else prepare_dt<LBM_F16S, false, GEN>(c);
+            if (c->sr) prepare_dt<LBM_F16S, true, GEN, false>(c);
+            else prepare_dt<LBM_F16S, false, GEN, false>(c);
     }
 }
 
 cudaError_t prepare_step(lbm_ctx* c) {
-    if (c->gen) prepare_model<true>(c);
+    if (hybrid_inc(c)) prepare_dt<LBM_F64, false, false, true>(c);
+    else if (c->gen) prepare_model<true>(c);
     else prepare_model<false>(c);
     return cudaGetLastError();
 }

@@ -128,7 +128,7 @@ void free_all(lbm_ctx* c) {
     drop_graphs(c);
     void* bufs[] = {c->tile_map, c->non_empty, c->nbr,    c->smask,  c->tflags, c->ntype,    c->nword,
                     c->groups,   c->fword,     c->fidx,   c->gfield, c->gfield_c, c->f[0], c->f[1],
-                    c->partials, c->d_out, c->seed, c->tlane, c->nrec, c->frank, c->check};
+                    c->partials, c->d_out, c->seed, c->tlane, c->nrec, c->frank, c->check, c->run_tables};
     for (void* b : bufs)
         if (b) lbm::dfree(b);
     c->tile_map = nullptr;
@@ -144,6 +144,8 @@ void free_all(lbm_ctx* c) {
     c->tlane = nullptr;
     c->nrec = nullptr;
     c->frank = nullptr;
+    c->run_tables = nullptr;
+    c->fsrc = nullptr;
     c->gfield_c = nullptr;
     c->f[0] = c->f[1] = nullptr;
     c->gfield = nullptr;
@@ -510,6 +512,27 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
             LBM_CREATE_CUDA(e);
             LBM_CREATE_CUDA(e2);
         }
+        c->p.n_padded = c->n_sgroups * lbm::GROUP_LANES;
+        if (dtype == LBM_F16S && !groups.empty() && lbm::idx32(c)) {
+            // import lists and staged offsets of the FP16 step (lbm_internal.cuh), one buffer
+            const size_t src = 0, src8 = src + (size_t)lanes * 32, imp = (src8 + (size_t)lanes * 4 + 15) / 16 * 16,
+                         ent = (imp + groups.size() * sizeof(int2) + 15) / 16 * 16;
+            LBM_CREATE_CUDA(lbm::dmalloc(&c->run_tables, ent + groups.size() * (size_t)lbm::GROUP_MAX_IMPORTS * 4));
+            char* b = static_cast<char*>(c->run_tables);
+            c->fsrc = reinterpret_cast<uint4*>(b + src);
+            c->fsrc8 = reinterpret_cast<uint32_t*>(b + src8);
+            c->imports = reinterpret_cast<int2*>(b + imp);
+            c->entries = reinterpret_cast<uint32_t*>(b + ent);
+            LBM_CREATE_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
+            LBM_CREATE_CUDA(lbm::launch_imports(c, d_bad));
+            LBM_CREATE_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, c->stream));
+            LBM_CREATE_CUDA(cudaStreamSynchronize(c->stream));
+            if (bad) {   // a group with too many imports: the step pulls node by node
+                lbm::dfree(c->run_tables);
+                c->run_tables = nullptr;
+                c->fsrc = nullptr;
+            }
+        }
         LBM_CREATE_CUDA(cudaStreamSynchronize(c->stream));
     }
     c->p.omega = 1.0;
@@ -517,7 +540,6 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
     c->p.rho_out = 1.0;
     c->p.n_tiles = c->n_tiles;
     c->p.n_lanes = c->n_own_nonsolid;
-    c->p.n_padded = c->n_sgroups * lbm::GROUP_LANES;
     c->p.check = c->check;
     cleanup();
 #undef LBM_CREATE_CUDA

@@ -45,6 +45,14 @@
 //                               five directions per word (rank_of); 0 for a bounced link.
 //                               f_i(x - c_i) then lives at nrec[tile][nb] + 256 i + rank
 //   gfield_c [n_fluid]           the per-node force in the same order
+// FP16 storage, when no work group has more than GROUP_MAX_IMPORTS pulls from other groups and
+// the indices fit 32 bits (else NULL, and the step pulls node by node):
+//   imports  [n_groups] int2     {first entry, entries} of each work group
+//   entries  [n_groups][1536] uint32   the aligned 32-bit word of a copy that holds an import's
+//                               value, in direction order, each list padded to a multiple of 4
+//   fsrc     [n_fluid][2] uint4, fsrc8 [n_fluid] uint32   per node and direction 1..18 the 16-bit
+//                               byte offset of its value in the staged group: (256 i + lane) * 2
+//                               in its own data blocks, 9728 + 4 k + (0 or 2) for import k
 #pragma once
 
 #include <cuda_runtime.h>
@@ -78,6 +86,7 @@ constexpr int STEP_RW = 2;          // read and write each node's own values ("r
 constexpr int GROUP_MAX_NODES = 256;       // work-group size of the 4-byte-or-smaller formats
 constexpr int GROUP_MAX_NODES_F64 = 256;   // and of FP64 storage (see the step kernel's CTA shape)
 constexpr int GROUP_LANES = 256;           // lanes of a storage group: the length of its data blocks
+constexpr int GROUP_MAX_IMPORTS = 1536;    // imports of a work group the FP16 step can stage
 constexpr int FLAG_HAS_BC = 1;
 // F16S storage scale: h is stored as half(h * 2^12), so |h| in [1.5e-8, 16] is normal.
 constexpr float F16_SCALE = 4096.0f;
@@ -236,6 +245,11 @@ struct lbm_ctx {
     int32_t* tlane = nullptr;
     int64_t* nrec = nullptr;
     uint4* frank = nullptr;
+    void* run_tables = nullptr;   // the buffer of the four below; fsrc NULL: not in use
+    uint4* fsrc = nullptr;
+    uint32_t* fsrc8 = nullptr;
+    int2* imports = nullptr;
+    uint32_t* entries = nullptr;
     int64_t n_sgroups = 0;      // storage groups of a copy (work groups and ghost-plane groups)
     void* gfield_c = nullptr;
     int64_t n_groups = 0;
@@ -279,6 +293,7 @@ cudaError_t launch_tile_meta(lbm_ctx* c, const uint8_t* nt);
 cudaError_t launch_node_words(lbm_ctx* c);
 cudaError_t launch_lane_lists(lbm_ctx* c, const int64_t* lane0, const uint8_t* lt);
 cudaError_t launch_node_records(lbm_ctx* c);
+cudaError_t launch_imports(lbm_ctx* c, int* too_many);
 cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]);
 // chained: the launch directly before on the stream is a step or adjoint launch of the same
 // call (lbm_async.cuh).

@@ -251,46 +251,16 @@ __device__ __forceinline__ void store_f16_conserving(const float v[Q], __half* _
     put(0, v[0] + m);
 }
 
-// Read this thread's staged values of group g into registers, let `next` issue the
-// gathers of the thread's node in the next group into the same column, then collide
-// and store. A thread without a node in g still calls next.
-template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, typename Next>
-__device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int dslot, const int4 h, int64_t sg,
-                                              typename Store<DT>::T* __restrict__ B, const StepParams& p,
-                                              bool has_gf, uint32_t key, Next&& next) {
+// Boundary handling, collision and store of one node of work group g (storage group sg), from its
+// 19 gathered values; w its word, Fx its x force.
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC>
+__device__ __forceinline__ void finish_node(typename Store<DT>::R v[Q], uint32_t w, typename Store<DT>::R Fx, const int4 h,
+                                            int64_t sg, typename Store<DT>::T* __restrict__ B, const StepParams& p,
+                                            bool has_gf, uint32_t key) {
     using R = typename Store<DT>::R;
-    using T = typename Store<DT>::T;
     const int t = threadIdx.x;
-    const uint32_t w = sm.word[mslot][t];
     const int type = (int)((w >> WORD_TYPE_SHIFT) & 3u);
-    if (type == LBM_SOLID) {
-        next(0u);
-        return;
-    }
     const int lt = (int)((w >> WORD_LT_SHIFT) & (uint32_t)WORD_LT_MASK), s = (int)((w >> WORD_SLOT_SHIFT) & 63u);
-    R v[Q];
-    const uint32_t odd = DT == LBM_F16S ? sm.odd[dslot][DT == LBM_F16S ? t : 0] : 0u;
-    uint32_t fold = 0;
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        if constexpr (DT == LBM_F16S) {
-            const uint32_t word = (uint32_t)sm.data[dslot][i][t];
-            fold ^= word;
-            // both halves converted, the wanted one selected (2 % faster than shifting the
-            // word by the half's offset first); the value is to_arith's
-            const __half2 h2 = *reinterpret_cast<const __half2*>(&word);
-            const float lo = __low2float(h2), hi = __high2float(h2);
-            v[i] = ((odd >> i) & 1u ? hi : lo) * F16_INV_SCALE;
-        } else {
-            const typename Staged<DT>::E raw = sm.data[dslot][i][t];
-            fold ^= (uint32_t)raw;
-            v[i] = to_arith<DT>(*reinterpret_cast<const T*>(&raw), i);
-        }
-    }
-    // one slot: 0 (p.zero is 0, unknown to the compiler), but only once every value above
-    // has arrived in its register
-    next(StepCfg<DT>::SLOTS == 1 ? fold & p.zero : 0u);
-    const R Fx = has_gf ? sm.gf[mslot][t] : par<R>(p.g[0], p.g_f[0]);
     const R Fy = par<R>(p.g[1], p.g_f[1]), Fz = par<R>(p.g[2], p.g_f[2]);
     if (MODE == STEP_FULL && ((w >> WORD_LID_BIT) & 1u)) {
         // moving wall: bounced links that cross the lid face gain 6 w_i (c_i . u_lid)
@@ -350,6 +320,48 @@ __device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int d
 #pragma unroll
         for (int i = 0; i < Q; i++) B[own + i * GROUP_LANES] = to_store<DT>(v[i], i);
     }
+}
+
+// Read this thread's staged values of group g into registers, let `next` issue the
+// gathers of the thread's node in the next group into the same column, then collide
+// and store. A thread without a node in g still calls next.
+template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, typename Next>
+__device__ __forceinline__ void compute_store(StepSmem<DT>& sm, int mslot, int dslot, const int4 h, int64_t sg,
+                                              typename Store<DT>::T* __restrict__ B, const StepParams& p,
+                                              bool has_gf, uint32_t key, Next&& next) {
+    using R = typename Store<DT>::R;
+    using T = typename Store<DT>::T;
+    const int t = threadIdx.x;
+    const uint32_t w = sm.word[mslot][t];
+    const int type = (int)((w >> WORD_TYPE_SHIFT) & 3u);
+    if (type == LBM_SOLID) {
+        next(0u);
+        return;
+    }
+    R v[Q];
+    const uint32_t odd = DT == LBM_F16S ? sm.odd[dslot][DT == LBM_F16S ? t : 0] : 0u;
+    uint32_t fold = 0;
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+        if constexpr (DT == LBM_F16S) {
+            const uint32_t word = (uint32_t)sm.data[dslot][i][t];
+            fold ^= word;
+            // both halves converted, the wanted one selected (2 % faster than shifting the
+            // word by the half's offset first); the value is to_arith's
+            const __half2 h2 = *reinterpret_cast<const __half2*>(&word);
+            const float lo = __low2float(h2), hi = __high2float(h2);
+            v[i] = ((odd >> i) & 1u ? hi : lo) * F16_INV_SCALE;
+        } else {
+            const typename Staged<DT>::E raw = sm.data[dslot][i][t];
+            fold ^= (uint32_t)raw;
+            v[i] = to_arith<DT>(*reinterpret_cast<const T*>(&raw), i);
+        }
+    }
+    // one slot: 0 (p.zero is 0, unknown to the compiler), but only once every value above
+    // has arrived in its register
+    next(StepCfg<DT>::SLOTS == 1 ? fold & p.zero : 0u);
+    finish_node<DT, VAR, MODE, GEN, XF, INC>(v, w, has_gf ? sm.gf[mslot][t] : par<R>(p.g[0], p.g_f[0]), h, sg, B, p,
+                                             has_gf, key);
 }
 
 static_assert(LBM_INLET == 2 && LBM_OUTLET == 3, "closure_df takes the node types by value");
@@ -443,6 +455,147 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
     cp_async_wait<0>();
 }
 
+// ------------------------------------------------- FP16 storage: the group's blocks staged whole
+// A work group's 19 data blocks are one run of 9 728 bytes in FP16, and on the porous pack 75 %
+// of its pulls come from that run: it is copied into shared memory whole, in 16-byte pieces, and
+// only the pulls from other groups (4.6 a node) are gathered, by the group's list of imports,
+// one aligned 32-bit word each. A node then reads its 19 values from shared memory at 16-bit
+// offsets precomputed at creation (fsrc: own block or import, the half of an import's word, its
+// own opposite direction for a bounced link), with two instructions a value. The per-node
+// pulls of k_step, forming 18 addresses and selecting the half of each staged word, were a
+// third of the FP16 step (233 us on the porous 256^3 pack, 156 us without them), which issues
+// 66 % of cycles; the lists cost 32 bytes a node more than the ranks, which FP16, at 44 % of
+// the DRAM rate, has room for. (FP32 and FP64 are nearer to the DRAM rate and keep the pulls.)
+// Measured: 188 us (25.1 -> 31.2 GLUPS); 190^3 cavity 1.24 times, 32^3 channel 1.05 times as fast.
+constexpr int RUN_BYTES = Q * GROUP_LANES * 2;
+constexpr int RUN_CHUNKS = RUN_BYTES / 16;
+struct RunSmem {
+    int4 hdr[4];                                        // {t0, tiles, f0, nodes}
+    int2 imp[4];                                        // {first import, imports}
+    // two buffers: the group's run, then its imports' words
+    unsigned char data[2][RUN_BYTES + 4 * GROUP_MAX_IMPORTS];
+    uint4 entry[GROUP_MAX_IMPORTS / 4];                 // source words of the next group's imports
+    uint4 src[2][GROUP_LANES];                          // fsrc of the node, own thread
+    uint32_t src8[GROUP_LANES];
+    uint32_t word[GROUP_LANES];
+    float gf[GROUP_LANES];                              // last (see StepSmem)
+};
+
+template <bool VAR, int MODE, bool GEN>
+__global__ void __launch_bounds__(GROUP_LANES, 4)
+k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __restrict__ groups,
+           const int2* __restrict__ imports, const uint32_t* __restrict__ entries, const uint4* __restrict__ fsrc,
+           const uint32_t* __restrict__ fsrc8, const uint32_t* __restrict__ fword, const float* __restrict__ gfield_c,
+           int64_t n_groups, StepParams p, const uint32_t* __restrict__ seed_in, uint32_t* __restrict__ seed_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RunSmem& sm = *reinterpret_cast<RunSmem*>(smem_raw);
+    constexpr int DT = LBM_F16S;
+    const int t = threadIdx.x;
+    const int64_t G = gridDim.x;
+    const int64_t g0 = G - 1 - blockIdx.x;   // as in k_step
+    const bool has_gf = gfield_c != nullptr;
+    const auto header = [&](int it) { return group_header<DT>(sm.hdr[it & 3], p); };
+    const auto issue_header = [&](int it) {
+        const int64_t g = g0 + it * G;
+        if (t == 0 && g < n_groups) {
+            cp_async16(&sm.hdr[it & 3], groups + g);
+            cp_async8(&sm.imp[it & 3], imports + g);
+        }
+    };
+    // the imports' source words: thread t reads and later uses entries 4 t ... 4 t + 3 (+ 1024)
+    const auto issue_entries = [&](int it) {
+        if (MODE == STEP_RW || g0 + it * G >= n_groups) return;
+        const int2 m = sm.imp[it & 3];
+        for (int k = t; 4 * k < m.y; k += GROUP_LANES) cp_async16(&sm.entry[k], entries + m.x + 4 * k);
+    };
+    const auto issue_data = [&](int it) {
+        const int64_t g = g0 + it * G;
+        if (g >= n_groups) return;
+        unsigned char* d = sm.data[it & 1];
+        const char* run = reinterpret_cast<const char*>(A + (p.sg0 + g) * (Q * GROUP_LANES));
+        for (int k = t; k < RUN_CHUNKS; k += GROUP_LANES) cp_async16(d + 16 * k, run + 16 * k);
+        if (MODE == STEP_RW) return;
+        const int n = sm.imp[it & 3].y;
+        for (int k = t; 4 * k < n; k += GROUP_LANES) {
+            const uint4 e = sm.entry[k];
+            uint32_t* dst = reinterpret_cast<uint32_t*>(d + RUN_BYTES) + 4 * k;
+            const uint32_t word[4] = {e.x, e.y, e.z, e.w};   // the list is padded to fours
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (check_ok(2 * (int64_t)word[j] < p.n_padded * Q, CHECK_NEIGHBOUR, g, p))
+                    cp_async4(dst + j, reinterpret_cast<const uint32_t*>(A) + word[j]);
+        }
+    };
+    // zero, computed from values just read (dep), orders the copies after the reads
+    const auto issue_own = [&](int it, uint32_t dep) {
+        const int64_t g = g0 + it * G;
+        if (g >= n_groups) return;
+        const int4 h = header(it);
+        if (t < h.w) {
+            const int64_t n = (int64_t)h.z + t;
+            const int o = t + (int)dep;
+            cp_async4(&sm.word[o], fword + n);
+            cp_async16(&sm.src[0][o], fsrc + 2 * n);
+            cp_async16(&sm.src[1][o], fsrc + 2 * n + 1);
+            cp_async4(&sm.src8[o], fsrc8 + n);
+            if (has_gf) cp_async4(&sm.gf[o], gfield_c + n);
+        } else {
+            sm.word[t] = 0;
+        }
+    };
+    // a thread without a node reads by the offsets it finds: valid ones from the start
+    sm.src[0][t] = sm.src[1][t] = make_uint4(0u, 0u, 0u, 0u);
+    sm.src8[t] = 0u;
+    for (int k = 0; k < 3; k++) issue_header(k);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    issue_entries(0);
+    issue_own(0, 0u);
+    cp_async_commit();
+    cp_async_wait<0>();
+    grid_wait();   // the tables above are constant; from here on the launch before is complete
+    uint32_t key = 0;
+    if (VAR) {
+        // step counter of the rounding hash, as in k_step
+        const uint32_t c = __ldcg(seed_in);
+        if (blockIdx.x == 0 && t == 0) *seed_out = c + 1u;
+        key = fmix32(c * 0x9e3779b9u + 0x7f4a7c15u);
+    }
+    issue_data(0);
+    issue_entries(1);
+    cp_async_commit();
+    int it = 0;
+    for (int64_t g = g0; g < n_groups; g += G, it++) {
+        cp_async_wait<0>();
+        __syncthreads();   // data(it), header(it + 2) visible; iteration it - 1 finished
+        issue_data(it + 1);
+        issue_entries(it + 2);
+        issue_header(it + 3);
+        cp_async_commit();
+        const int4 h = header(it);
+        const uint32_t w = sm.word[t];
+        const uint4 s0 = sm.src[0][t], s1 = sm.src[1][t];
+        const uint32_t s8 = sm.src8[t];
+        const float Fx = has_gf ? sm.gf[t] : p.g_f[0];
+        const uint32_t off[9] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w, s8};
+        const unsigned char* d = sm.data[it & 1];
+        float v[Q];
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            uint32_t o = (uint32_t)(i * GROUP_LANES + t) * 2u;
+            if (MODE != STEP_RW && i > 0) o = (i & 1) ? off[(i - 1) >> 1] & 0xffffu : off[(i - 1) >> 1] >> 16;
+            if (!check_ok(o < sizeof(sm.data[0]), CHECK_NEIGHBOUR, (int64_t)h.z + t, p)) o = 0;
+            v[i] = to_arith<DT>(*reinterpret_cast<const __half*>(d + o), i);
+        }
+        issue_own(it + 1, (w ^ s0.x ^ s0.y ^ s0.z ^ s0.w ^ s1.x ^ s1.y ^ s1.z ^ s1.w ^ s8 ^ __float_as_uint(Fx)) & p.zero);
+        cp_async_commit();
+        if (((w >> WORD_TYPE_SHIFT) & 3u) != LBM_SOLID)
+            finish_node<DT, VAR, MODE, GEN, false, false>(v, w, Fx, h, p.sg0 + g, B, p, has_gf, key);
+    }
+    cp_async_wait<0>();
+}
+
 // Shared memory of a launch: the whole StepSmem with a per-node force field, without its
 // force staging (the last member) otherwise.
 template <int DT>
@@ -478,6 +631,35 @@ static int step_grid(int64_t n_groups, bool with_gf) {
         ps = std::max(1, std::min(ps, step_ctas<DT, GEN>()));
     }
     return (int)std::max<int64_t>(1, std::min<int64_t>(n_groups, (int64_t)ps * n_sm));
+}
+
+// Persistent grid of the FP16 step on staged runs.
+template <bool VAR, int MODE, bool GEN>
+static int run_grid(int64_t n_groups, bool with_gf) {
+    static int per_sm[2] = {-1, -1}, n_sm = 0;
+    int& ps = per_sm[with_gf ? 1 : 0];
+    if (ps < 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RunSmem));
+        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_step_run<VAR, MODE, GEN>, GROUP_LANES,
+                                                      with_gf ? sizeof(RunSmem) : offsetof(RunSmem, gf));
+        ps = std::max(1, std::min(ps, 4));
+    }
+    return (int)std::max<int64_t>(1, std::min<int64_t>(n_groups, (int64_t)ps * n_sm));
+}
+
+template <bool VAR, int MODE, bool GEN>
+static cudaError_t launch_run(lbm_ctx* c, const void* A, void* B, bool chained) {
+    const bool with_gf = c->gfield != nullptr;
+    const int from = A == c->f[0] ? 0 : 1;
+    return launch_chained(k_step_run<VAR, MODE, GEN>, (unsigned)run_grid<VAR, MODE, GEN>(c->n_groups, with_gf),
+                          (unsigned)GROUP_LANES, with_gf ? sizeof(RunSmem) : offsetof(RunSmem, gf), c->stream, chained,
+                          (const __half*)A, (__half*)B, c->groups, c->imports, c->entries, c->fsrc, c->fsrc8, c->fword,
+                          with_gf ? (const float*)c->gfield_c : nullptr, c->n_groups, c->p,
+                          c->seed ? c->seed + from : nullptr, c->seed ? c->seed + (1 - from) : nullptr);
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
@@ -541,6 +723,7 @@ static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B, bool ch
                                : launch_step_dt<LBM_F64, false, MODE, GEN, false>(c, A, B, chained);
         case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN, false>(c, A, B, chained);
         default:
+            if (c->fsrc) return c->sr ? launch_run<true, MODE, GEN>(c, A, B, chained) : launch_run<false, MODE, GEN>(c, A, B, chained);
             return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN, false>(c, A, B, chained)
                          : launch_step_dt<LBM_F16S, false, MODE, GEN, false>(c, A, B, chained);
     }
@@ -569,6 +752,11 @@ static void prepare_model(lbm_ctx* c) {
             break;
         case LBM_F32: prepare_dt<LBM_F32, false, GEN, false>(c); break;
         default:
+            if (c->fsrc) {
+                if (c->sr) run_grid<true, STEP_FULL, GEN>(1, c->gfield != nullptr);
+                else run_grid<false, STEP_FULL, GEN>(1, c->gfield != nullptr);
+                break;
+            }
             if (c->sr) prepare_dt<LBM_F16S, true, GEN, false>(c);
             else prepare_dt<LBM_F16S, false, GEN, false>(c);
     }

@@ -342,6 +342,83 @@ cudaError_t launch_node_records(lbm_ctx* c) {
     return cudaGetLastError();
 }
 
+// Import lists and staged offsets of FP16 storage, one CTA per work group, one thread per node.
+// A group's imports (pulls whose source lies in another storage group) are numbered direction by
+// direction and lane by lane, so that a direction's imports read runs of other groups' blocks; a
+// group with more than fit its list sets *too_many.
+__global__ void __launch_bounds__(GROUP_LANES) k_imports(const int4* __restrict__ groups, const uint32_t* __restrict__ fword,
+                                                         const uint32_t* __restrict__ fidx, const int32_t* __restrict__ nbr,
+                                                         const uint64_t* __restrict__ smask,
+                                                         const int32_t* __restrict__ tlane, int64_t sg0,
+                                                         int* __restrict__ too_many, int2* __restrict__ imports, uint32_t* __restrict__ entries,
+                                                         uint32_t* __restrict__ fsrc, uint32_t* __restrict__ fsrc8) {
+    __shared__ int warp_n[GROUP_LANES / 32];
+    const int64_t g = blockIdx.x;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int4 h = groups[g];
+    const bool on = t < h.w;
+    const int64_t n = (int64_t)h.z + t;
+    uint32_t w = 0, gi = 0;
+    if (on) {
+        w = fword[n];
+        gi = fidx[n];
+    }
+    const int64_t k = gi >> 6;
+    const int s = (int)(gi & 63u), x = s & 3, y = (s >> 2) & 3, z = s >> 4;
+    const uint32_t base = (uint32_t)(sg0 + g);
+    uint32_t* list = entries + g * GROUP_MAX_IMPORTS;
+    int count = 0;   // imports of the directions so far
+    uint32_t off[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int i = 1; i < Q; i++) {
+        uint32_t o = (uint32_t)(inv(i) * GROUP_LANES + t) * 2u, P = 0;
+        bool import = false;
+        if (on && !((w >> i) & 1u)) {
+            const int sx = x - cx(i), sy = y - cy(i), sz = z - cz(i);
+            const int nb = 13 + (sx >> 2) + 3 * (sy >> 2) + 9 * (sz >> 2);
+            const int ss = (sx & 3) | ((sy & 3) << 2) | ((sz & 3) << 4);
+            const int32_t r = nbr[k * NBR_STRIDE + nb];   // >= 0: the link does not bounce
+            P = node_lane((uint32_t)tlane[r], smask[r], ss);
+            import = P / GROUP_LANES != base;
+            o = (uint32_t)(i * GROUP_LANES + (P % GROUP_LANES)) * 2u;
+        }
+        const uint32_t b = __ballot_sync(0xffffffffu, import);
+        if (lane == 0) warp_n[warp] = __popc(b);
+        __syncthreads();
+        int before = count;
+        for (int v = 0; v < GROUP_LANES / 32; v++) {
+            if (v < warp) before += warp_n[v];
+            count += warp_n[v];
+        }
+        __syncthreads();
+        if (import) {
+            const int slot = before + __popc(b & ((1u << lane) - 1u));
+            const int64_t e = data_index(P, i);
+            if (slot < GROUP_MAX_IMPORTS) list[slot] = (uint32_t)(e >> 1);
+            o = (uint32_t)(Q * GROUP_LANES * 2 + 4 * slot) + 2u * (uint32_t)(e & 1);
+        }
+        off[(i - 1) >> 1] |= (i & 1) ? o : o << 16;
+    }
+    if (count > GROUP_MAX_IMPORTS) {
+        if (t == 0) *too_many = 1;
+        return;
+    }
+    if (t == 0) imports[g] = make_int2((int)(g * GROUP_MAX_IMPORTS), count);
+    if (t < (4 - (count & 3)) % 4) list[count + t] = 0;   // padding: word 0 of the copy
+    if (on) {
+#pragma unroll
+        for (int j = 0; j < 8; j++) fsrc[n * 8 + j] = off[j];
+        fsrc8[n] = off[8];
+    }
+}
+
+cudaError_t launch_imports(lbm_ctx* c, int* too_many) {
+    k_imports<<<(unsigned)c->n_groups, GROUP_LANES, 0, c->stream>>>(c->groups, c->fword, c->fidx, c->nbr, c->smask, c->tlane,
+                                                                   c->p.sg0, too_many, c->imports, c->entries,
+                                                                   reinterpret_cast<uint32_t*>(c->fsrc), c->fsrc8);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]) {
     const unsigned g = std::min(grid_for(c->n_tiles * SLOTS, 256), 152u * 8u);
     switch (c->dtype) {

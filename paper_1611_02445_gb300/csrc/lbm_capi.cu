@@ -88,6 +88,28 @@ cudaError_t dev_alloc(T** p, size_t count) {
     return lbm::dmalloc(reinterpret_cast<void**>(p), count * sizeof(T));
 }
 
+// Several arrays in one device allocation (each one costs 50 to 100 us to make and again to
+// release): `add` the arrays, then `alloc` sets their pointers, 256-byte aligned.
+struct Arrays {
+    struct Part {
+        void** p;
+        size_t at;
+    };
+    Part parts[8];   // add at most eight
+    int n = 0;
+    size_t size = 0;
+    template <typename T> void add(T** p, size_t count) {
+        parts[n++] = {reinterpret_cast<void**>(p), size};
+        size += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+    }
+    cudaError_t alloc(void** base) {
+        const cudaError_t e = lbm::dmalloc(base, std::max<size_t>(size, 1));
+        if (e == cudaSuccess)
+            for (int k = 0; k < n; k++) *parts[k].p = static_cast<char*>(*base) + parts[k].at;
+        return e;
+    }
+};
+
 void drop_graphs(lbm_ctx* c) {
     for (int i = 0; i < 2; i++)
         if (c->graph[i]) {
@@ -126,13 +148,14 @@ cudaError_t build_graph(lbm_ctx* c, int start) {
 
 void free_all(lbm_ctx* c) {
     drop_graphs(c);
-    void* bufs[] = {c->tile_map, c->non_empty, c->nbr,    c->smask,  c->tflags, c->ntype,    c->nword,
-                    c->groups,   c->fword,     c->fidx,   c->gfield, c->gfield_c, c->f[0], c->f[1],
-                    c->partials, c->d_out, c->seed, c->tlane, c->nrec, c->frank, c->check, c->run_tables};
+    void* bufs[] = {c->tile_map, c->non_empty, c->tile_tables, c->node_tables, c->gfield, c->gfield_c, c->f[0], c->f[1],
+                    c->partials, c->d_out,     c->seed,        c->check,       c->run_tables};
     for (void* b : bufs)
         if (b) lbm::dfree(b);
     c->tile_map = nullptr;
     c->non_empty = nullptr;
+    c->tile_tables = nullptr;
+    c->node_tables = nullptr;
     c->nbr = nullptr;
     c->smask = nullptr;
     c->tflags = nullptr;
@@ -296,16 +319,14 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
     c->stream = static_cast<cudaStream_t>(stream);
 
     uint8_t* d_nt = nullptr;
+    void* scratch = nullptr;   // the buffer of the four below
     uint8_t* d_flag = nullptr;
     int64_t* d_sums = nullptr;
     int64_t* d_count = nullptr;
     int* d_bad = nullptr;
     auto cleanup = [&]() {
         if (!on_device && d_nt) lbm::dfree(d_nt);
-        if (d_flag) lbm::dfree(d_flag);
-        if (d_sums) lbm::dfree(d_sums);
-        if (d_count) lbm::dfree(d_count);
-        if (d_bad) lbm::dfree(d_bad);
+        if (scratch) lbm::dfree(scratch);
     };
     auto bail = [&](lbm_status s2) {
         g_create_err = c->err.empty() ? std::string("lbm_create failed") : c->err;
@@ -330,10 +351,14 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
     const int64_t nb = lbm::scan_block_count(nT);
     LBM_CREATE_CUDA(dev_alloc(&c->tile_map, (size_t)nT));
     LBM_CREATE_CUDA(dev_alloc(&c->non_empty, (size_t)nT));
-    LBM_CREATE_CUDA(dev_alloc(&d_flag, (size_t)nT));
-    LBM_CREATE_CUDA(dev_alloc(&d_sums, (size_t)nb));
-    LBM_CREATE_CUDA(dev_alloc(&d_count, 1));
-    LBM_CREATE_CUDA(dev_alloc(&d_bad, 1));
+    {
+        Arrays tmp;
+        tmp.add(&d_flag, (size_t)nT);
+        tmp.add(&d_sums, (size_t)nb);
+        tmp.add(&d_count, 1);
+        tmp.add(&d_bad, 1);
+        LBM_CREATE_CUDA(tmp.alloc(&scratch));
+    }
     LBM_CREATE_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
     LBM_CREATE_CUDA(lbm::launch_tile_flags(d_nt, nx, ny, nz, c->Tx, c->Ty, c->Tz, d_flag, d_bad, c->stream));
     LBM_CREATE_CUDA(lbm::launch_scan_flags(d_flag, nT, c->tile_map, c->non_empty, d_count, d_sums, nb, c->stream));
@@ -357,11 +382,15 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
     }
     c->n_tiles = count;
     c->n_partials = lbm::reduce_blocks(count);
-    LBM_CREATE_CUDA(dev_alloc(&c->nbr, (size_t)count * lbm::NBR_STRIDE));
-    LBM_CREATE_CUDA(dev_alloc(&c->nword, (size_t)count * lbm::SLOTS));
-    LBM_CREATE_CUDA(dev_alloc(&c->smask, (size_t)count));
-    LBM_CREATE_CUDA(dev_alloc(&c->tflags, (size_t)count));
-    LBM_CREATE_CUDA(dev_alloc(&c->ntype, (size_t)count * lbm::SLOTS));
+    {
+        Arrays tables;
+        tables.add(&c->nbr, (size_t)count * lbm::NBR_STRIDE);
+        tables.add(&c->nword, (size_t)count * lbm::SLOTS);
+        tables.add(&c->smask, (size_t)count);
+        tables.add(&c->tflags, (size_t)count);
+        tables.add(&c->ntype, (size_t)count * lbm::SLOTS);
+        LBM_CREATE_CUDA(tables.alloc(&c->tile_tables));
+    }
     LBM_CREATE_CUDA(dev_alloc(&c->partials, (size_t)c->n_partials * 4));
     LBM_CREATE_CUDA(dev_alloc(&c->d_out, 8));
 #ifdef LBM_CHECKED
@@ -482,12 +511,16 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
         // state depends on the populations alone
         LBM_CREATE_CUDA(cudaMemsetAsync(c->f[0], 0, copy_bytes, c->stream));
         LBM_CREATE_CUDA(cudaMemsetAsync(c->f[1], 0, copy_bytes, c->stream));
-        LBM_CREATE_CUDA(dev_alloc(&c->tlane, (size_t)std::max<int64_t>(count, 1)));
-        LBM_CREATE_CUDA(dev_alloc(&c->nrec, (size_t)std::max<int64_t>(count, 1) * lbm::NBR_STRIDE));
-        LBM_CREATE_CUDA(dev_alloc(&c->groups, groups.size()));
-        LBM_CREATE_CUDA(dev_alloc(&c->fword, (size_t)lanes));
-        LBM_CREATE_CUDA(dev_alloc(&c->fidx, (size_t)lanes));
-        LBM_CREATE_CUDA(dev_alloc(&c->frank, (size_t)lanes));
+        {
+            Arrays tables;
+            tables.add(&c->tlane, (size_t)count);
+            tables.add(&c->nrec, (size_t)count * lbm::NBR_STRIDE);
+            tables.add(&c->groups, groups.size());
+            tables.add(&c->fword, (size_t)lanes);
+            tables.add(&c->fidx, (size_t)lanes);
+            tables.add(&c->frank, (size_t)lanes);
+            LBM_CREATE_CUDA(tables.alloc(&c->node_tables));
+        }
         if (count > 0) {
             LBM_CREATE_CUDA(cudaMemcpyAsync(c->tlane, tlane_h.data(), tlane_h.size() * sizeof(int32_t),
                                             cudaMemcpyHostToDevice, c->stream));
@@ -496,8 +529,11 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
         if (!groups.empty()) {
             int64_t* d_lane0 = nullptr;
             uint8_t* d_lt = nullptr;
-            cudaError_t e = dev_alloc(&d_lane0, lane0.size());
-            if (e == cudaSuccess) e = dev_alloc(&d_lt, lt.size());
+            void* lists = nullptr;
+            Arrays tmp;
+            tmp.add(&d_lane0, lane0.size());
+            tmp.add(&d_lt, lt.size());
+            cudaError_t e = tmp.alloc(&lists);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(c->groups, groups.data(), groups.size() * sizeof(int4), cudaMemcpyHostToDevice,
                                     c->stream);
@@ -507,8 +543,7 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
                 e = cudaMemcpyAsync(d_lt, lt.data(), lt.size(), cudaMemcpyHostToDevice, c->stream);
             if (e == cudaSuccess) e = lbm::launch_lane_lists(c, d_lane0, d_lt);
             const cudaError_t e2 = cudaStreamSynchronize(c->stream);
-            lbm::dfree(d_lane0);
-            lbm::dfree(d_lt);
+            lbm::dfree(lists);
             LBM_CREATE_CUDA(e);
             LBM_CREATE_CUDA(e2);
         }

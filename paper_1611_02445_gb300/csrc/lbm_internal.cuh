@@ -234,6 +234,8 @@ struct lbm_ctx {
     cudaStream_t stream = nullptr;
     int32_t* tile_map = nullptr;
     uint32_t* non_empty = nullptr;
+    void* tile_tables = nullptr;   // the buffer of nbr, smask, tflags, ntype and nword
+    void* node_tables = nullptr;   // the buffer of groups, fword, fidx, tlane, nrec and frank
     int32_t* nbr = nullptr;
     uint64_t* smask = nullptr;
     uint32_t* tflags = nullptr;

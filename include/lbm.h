@@ -59,7 +59,8 @@ typedef enum {
  *                   Y = f^eq/tau + S runs in double-float (pairs of FP32, about 46-48
  *                   bits), because GB300's FP64 pipe has 2 lanes per SM. The equilibrium
  *                   inlet/outlet closures and the incompressible LBGK (lbm_set_model) use
- *                   the same arithmetic; MRT and the Zou-He completion run in FP64.
+ *                   the same arithmetic; MRT relaxes in FP64 from exact fixed-point
+ *                   moments, and the Zou-He completion runs in FP64.
  *                   Agrees with FP64 arithmetic to ~1e-14 relative per step.
  *   LBM_F64_NATIVE  FP64 storage, every operation of the step in FP64.
  *   LBM_F32         stores h_i = f_i - w_i as FP32 (the equilibrium-weight shift),

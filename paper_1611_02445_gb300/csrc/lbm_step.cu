@@ -27,7 +27,9 @@
 // stores of a group write whole 32-byte sectors (DRAM never reads a sector back to merge
 // a partial write), and a gather reads the source node at the neighbour record of its
 // tile plus the source slot's rank among that tile's non-solid slots (precomputed per
-// node and direction at creation).
+// node and direction at creation). FP16 storage takes k_step_run instead, which stages a
+// group's own blocks whole and gathers only what comes from other groups, unless a group has
+// more of that than its import list holds.
 #include <algorithm>
 #include <cmath>
 #include <cstddef>

@@ -272,6 +272,10 @@ __device__ __forceinline__ void finish_node(typename Store<DT>::R v[Q], uint32_t
     }
     if constexpr (MODE != STEP_FULL) {
         // calibration kernels: no collision, the gathered values are stored as they are
+    } else if constexpr (INC && DT == LBM_F32) {
+        // FP32 storage, incompressible LBGK
+        if (type == LBM_FLUID) collide<R, true, true>(v, LBM_FLUID, p, Fx, Fy, Fz);
+        else collide_model<R, true, false>(v, type, p, Fx, Fy, Fz);
     } else if constexpr (INC) {
         // FP64 storage, incompressible LBGK: the hybrid collision for fluid nodes (and Zou-He
         // boundary nodes once completed)
@@ -691,9 +695,10 @@ constexpr bool has_xf_form() {
     return DT == LBM_F64 && !VAR && MODE == STEP_FULL;
 }
 static bool force_along_x(const lbm_ctx* c) { return c->p.g[1] == 0.0 && c->p.g[2] == 0.0; }
-// The model with the hybrid collision's incompressible form.
-static bool hybrid_inc(const lbm_ctx* c) {
-    return c->dtype == LBM_F64 && !c->native64 && c->p.coll == LBM_COLL_BGK && c->p.eq == LBM_EQ_INCOMPR;
+// The formats with an incompressible LBGK kernel of their own, for contexts of that model.
+static bool own_inc(const lbm_ctx* c) {
+    return (c->dtype == LBM_F32 || (c->dtype == LBM_F64 && !c->native64)) && c->p.coll == LBM_COLL_BGK &&
+           c->p.eq == LBM_EQ_INCOMPR;
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool INC>
@@ -734,7 +739,9 @@ static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B, bool ch
 // The calibration kernels have no collision, so only the fused step has model variants.
 template <int MODE>
 static cudaError_t launch_step_mode(lbm_ctx* c, const void* A, void* B, bool chained) {
-    if (MODE == STEP_FULL && hybrid_inc(c)) return launch_step_dt<LBM_F64, false, STEP_FULL, false, true>(c, A, B, chained);
+    if (MODE == STEP_FULL && own_inc(c))
+        return c->dtype == LBM_F64 ? launch_step_dt<LBM_F64, false, STEP_FULL, false, true>(c, A, B, chained)
+                                   : launch_step_dt<LBM_F32, false, STEP_FULL, false, true>(c, A, B, chained);
     if (MODE == STEP_FULL && c->gen) return launch_step_model<STEP_FULL, true>(c, A, B, chained);
     return launch_step_model<MODE, false>(c, A, B, chained);
 }
@@ -765,7 +772,8 @@ static void prepare_model(lbm_ctx* c) {
 }
 
 cudaError_t prepare_step(lbm_ctx* c) {
-    if (hybrid_inc(c)) prepare_dt<LBM_F64, false, false, true>(c);
+    if (own_inc(c) && c->dtype == LBM_F64) prepare_dt<LBM_F64, false, false, true>(c);
+    else if (own_inc(c)) prepare_dt<LBM_F32, false, false, true>(c);
     else if (c->gen) prepare_model<true>(c);
     else prepare_model<false>(c);
     return cudaGetLastError();

@@ -111,7 +111,9 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_sum_partials(const double* __re
 
 // Density and momentum of the gathered populations: as in the collision, through sums and
 // differences of opposite directions; FP64 as exact integers in 2^-58 fixed point when every
-// population lies in [2^-6, 16) (no FP64 instruction), else in FP64.
+// population lies in [2^-6, 1) (no FP64 instruction), else in FP64. That bound keeps every sum
+// below 19, where the fixed point holds 32: a density of any size is accepted here (LBM_F64_NATIVE
+// steps it in FP64), and one of 3 or more has a rest population of 1 or more.
 template <typename R> __device__ __forceinline__ void pull_moments(const R v[Q], R& sum, R j[3]) {
     const R s = ((v[0] + (v[1] + v[3])) + ((v[2] + v[4]) + (v[5] + v[6]))) +
                 (((v[7] + v[9]) + (v[8] + v[10])) + ((v[11] + v[14]) + (v[12] + v[13]))) +
@@ -150,7 +152,7 @@ __device__ __forceinline__ R collide_adjoint(const R v[Q], R lam[Q], int type, c
         int64_t q[Q], fj[3];
         bool bad = false;
 #pragma unroll
-        for (int i = 0; i < Q; i++) q[i] = fix_from_double_fast(v[i], bad);
+        for (int i = 0; i < Q; i++) q[i] = fix_from_double_fast(v[i], bad, 5u);
         fix_moments(q, fix, fj[0], fj[1], fj[2]);
         D = fix_to_double(fix);
         for (int a = 0; a < 3; a++) j[a] = fix_to_double(fj[a]);

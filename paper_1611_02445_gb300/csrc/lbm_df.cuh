@@ -208,7 +208,7 @@ LBM_DF_HD int64_t fix_from_double(double d) {
 // pipe. Any other input (negative, below 2^-6, 16 or more, zero, not finite) sets `bad`
 // and returns an unspecified value; the caller then converts another way. Where this one
 // is valid the value is exact, so fix_from_double and fix_from_double_cvt give the same.
-// top: the largest shift taken; 6 narrows the range to 2^-6 <= d < 2.
+// top: the largest shift taken; 6 narrows the range to 2^-6 <= d < 2, 5 to 2^-6 <= d < 1.
 LBM_DF_HD int64_t fix_from_double_fast(double d, bool& bad, uint32_t top = 9u) {
     const uint64_t b = bits_of(d);
     const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;

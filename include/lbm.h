@@ -60,7 +60,8 @@ typedef enum {
  *                   bits), because GB300's FP64 pipe has 2 lanes per SM. The equilibrium
  *                   inlet/outlet closures and the incompressible LBGK (lbm_set_model) use
  *                   the same arithmetic; MRT relaxes in FP64 from exact fixed-point
- *                   moments, and the Zou-He completion runs in FP64.
+ *                   moments, and FP64 completes Zou-He nodes (and, in the incompressible
+ *                   LBGK, collides them).
  *                   Agrees with FP64 arithmetic to ~1e-14 relative per step.
  *   LBM_F64_NATIVE  FP64 storage, every operation of the step in FP64.
  *   LBM_F32         stores h_i = f_i - w_i as FP32 (the equilibrium-weight shift),

@@ -135,9 +135,9 @@ __device__ __forceinline__ void zou_he(R v[Q], int type, const StepParams& p) {
     }
 }
 
-// One node's collision, in place on v[19]. INC (a fluid node of a shifted format): the
-// incompressible equilibrium (Eq. 4, u = J), which is the form in J = j + F/2 with 1 in place of
-// 1 / rho. (Direction by direction in collide_model the FP32 step took 224 us on the porous 256^3
+// One node's collision, in place on v[19]. INC: the incompressible equilibrium (Eq. 4, u = J),
+// which is Eq. 3 with 1 in place of the density that multiplies u, and of 1 / rho in the form
+// in J = j + F/2. (Direction by direction in collide_model the FP32 step took 224 us on the porous 256^3
 // pack, 211 us so, in a kernel of its own: beside MRT in one kernel it cost that 1 %.)
 template <typename R, bool SHIFT, bool INC = false>
 __device__ __forceinline__ void collide(R v[Q], int type, const StepParams& p, R Fx, R Fy, R Fz) {
@@ -163,6 +163,7 @@ __device__ __forceinline__ void collide(R v[Q], int type, const StepParams& p, R
         rho = sum;
         D = sum;
     }
+    if (INC) rho = R(1);
     const R inv_rho = INC ? R(1) : R(1) / rho;
     const R Jx = jx + R(0.5) * Fx, Jy = jy + R(0.5) * Fy, Jz = jz + R(0.5) * Fz;
     const R ux = Jx * inv_rho;
@@ -211,6 +212,7 @@ __device__ __forceinline__ void collide(R v[Q], int type, const StepParams& p, R
             rq = par<R>(p.rho_out, p.rho_out_f);
             Dq = SHIFT ? par<R>(p.rho_out - 1.0, p.rho_out_m1_f) : rq;
         }
+        if (INC) rq = R(1);
         const R uu15 = R(1.5) * (ex * ex + ey * ey + ez * ez);
         v[0] = w0 * Dq - (w0 * rq) * uu15;
         eq_pair(v[1], v[3], w1, ex, Dq, rq, uu15);
@@ -290,30 +292,6 @@ __device__ __forceinline__ void relax_products(float v[Q], const float ve[Q], co
             if (mrt_row(k, i) != 0) acc += R(mrt_row(k, i)) * ms[k];
         v[i] = acc;
     }
-}
-
-// Equilibrium closure of an inlet or outlet node for the incompressible model in FP64 (Eq. 4):
-// w (rho + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u) with the node's density and u_in, or rho_out and the
-// node's u = j + F/2.
-__device__ __forceinline__ void closure_inc(double v[Q], int type, const StepParams& p, double Fx, double Fy, double Fz) {
-    double r = 0.0, ux = 0.5 * Fx, uy = 0.5 * Fy, uz = 0.5 * Fz;
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-        r += v[i];
-        if (cx(i)) ux += cx(i) > 0 ? v[i] : -v[i];
-        if (cy(i)) uy += cy(i) > 0 ? v[i] : -v[i];
-        if (cz(i)) uz += cz(i) > 0 ? v[i] : -v[i];
-    }
-    if (type == LBM_INLET) {
-        ux = p.u_in[0];
-        uy = p.u_in[1];
-        uz = p.u_in[2];
-    } else {
-        r = p.rho_out;
-    }
-    const double uu15 = 1.5 * (ux * ux + uy * uy + uz * uz);
-#pragma unroll
-    for (int i = 0; i < Q; i++) v[i] = feq_model<double>(i, r, 1.0, ux, uy, uz, uu15);
 }
 
 // MRT collision of a fluid node (Eq. 8), in place: v* = v + M^T t with

@@ -32,6 +32,7 @@ cudaError_t dmalloc(void** p, size_t bytes) {
     if (g_fail_after.load() >= 0 && g_fail_after.fetch_sub(1) == 0) return cudaErrorMemoryAllocation;
     const cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaSuccess) g_live_allocs.fetch_add(1);
+    else cudaGetLastError();   // returned here; left recorded, it would fail the next launch check
     return e;
 }
 

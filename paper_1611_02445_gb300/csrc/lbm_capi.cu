@@ -550,23 +550,28 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
         }
         c->p.n_padded = c->n_sgroups * lbm::GROUP_LANES;
         if (dtype == LBM_F16S && !groups.empty() && lbm::idx32(c)) {
-            // import lists and staged offsets of the FP16 step (lbm_internal.cuh), one buffer
+            // import lists and staged offsets of the FP16 step (lbm_internal.cuh), one buffer.
+            // They only make the step faster: without memory for them, or with a group that has
+            // more imports than its list holds, it pulls node by node.
             const size_t src = 0, src8 = src + (size_t)lanes * 32, imp = (src8 + (size_t)lanes * 4 + 15) / 16 * 16,
                          ent = (imp + groups.size() * sizeof(int2) + 15) / 16 * 16;
-            LBM_CREATE_CUDA(lbm::dmalloc(&c->run_tables, ent + groups.size() * (size_t)lbm::GROUP_MAX_IMPORTS * 4));
-            char* b = static_cast<char*>(c->run_tables);
-            c->fsrc = reinterpret_cast<uint4*>(b + src);
-            c->fsrc8 = reinterpret_cast<uint32_t*>(b + src8);
-            c->imports = reinterpret_cast<int2*>(b + imp);
-            c->entries = reinterpret_cast<uint32_t*>(b + ent);
-            LBM_CREATE_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
-            LBM_CREATE_CUDA(lbm::launch_imports(c, d_bad));
-            LBM_CREATE_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, c->stream));
-            LBM_CREATE_CUDA(cudaStreamSynchronize(c->stream));
-            if (bad) {   // a group with too many imports: the step pulls node by node
-                lbm::dfree(c->run_tables);
-                c->run_tables = nullptr;
-                c->fsrc = nullptr;
+            const cudaError_t e = lbm::dmalloc(&c->run_tables, ent + groups.size() * (size_t)lbm::GROUP_MAX_IMPORTS * 4);
+            if (e != cudaErrorMemoryAllocation) LBM_CREATE_CUDA(e);
+            if (e == cudaSuccess) {
+                char* b = static_cast<char*>(c->run_tables);
+                c->fsrc = reinterpret_cast<uint4*>(b + src);
+                c->fsrc8 = reinterpret_cast<uint32_t*>(b + src8);
+                c->imports = reinterpret_cast<int2*>(b + imp);
+                c->entries = reinterpret_cast<uint32_t*>(b + ent);
+                LBM_CREATE_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream));
+                LBM_CREATE_CUDA(lbm::launch_imports(c, d_bad));
+                LBM_CREATE_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(bad), cudaMemcpyDeviceToHost, c->stream));
+                LBM_CREATE_CUDA(cudaStreamSynchronize(c->stream));
+                if (bad) {
+                    lbm::dfree(c->run_tables);
+                    c->run_tables = nullptr;
+                    c->fsrc = nullptr;
+                }
             }
         }
         LBM_CREATE_CUDA(cudaStreamSynchronize(c->stream));

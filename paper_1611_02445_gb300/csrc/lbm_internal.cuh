@@ -45,8 +45,8 @@
 //                               five directions per word (rank_of); 0 for a bounced link.
 //                               f_i(x - c_i) then lives at nrec[tile][nb] + 256 i + rank
 //   gfield_c [n_fluid]           the per-node force in the same order
-// FP16 storage, when no work group has more than GROUP_MAX_IMPORTS pulls from other groups and
-// the indices fit 32 bits (else NULL, and the step pulls node by node):
+// FP16 storage, when no work group has more than GROUP_MAX_IMPORTS pulls from other groups, the
+// indices fit 32 bits and there is memory for them (else NULL, and the step pulls node by node):
 //   imports  [n_groups] int2     {first entry, entries} of each work group
 //   entries  [n_groups][1536] uint32   the aligned 32-bit word of a copy that holds an import's
 //                               value, in direction order, each list padded to a multiple of 4

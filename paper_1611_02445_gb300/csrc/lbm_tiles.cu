@@ -508,14 +508,33 @@ __device__ __forceinline__ void add_node_moments(const typename Store<DT>::T* __
     }
 }
 
-// FP64 mass and momentum. Per thread: FP64 storage adds its nodes' fixed-point moments in
-// 128-bit integers (exact), the other formats add pairs in FP32 and flush them into FP64
-// sums every RED_FLUSH nodes (before the rounding errors of the error sums matter); then a
-// warp shuffle tree, one partial per block and a fixed-order single-block pass. No atomics,
-// so the result depends only on the launch shape, which is fixed per context. The half
-// force is subtracted once per thread for a uniform force, and summed per node for a field.
+// FP64 mass and momentum. FP64 storage adds the nodes' fixed-point moments in 128-bit integers,
+// exactly, over a warp. The other formats add each node's pair to a triple of FP32 numbers, which
+// keeps the rounding errors of both parts, and that to FP64 sums every RED_FLUSH nodes. (A pair
+// carried over four nodes lost the last bits of small populations beside large ones: the
+// momentum of FP32 populations from 1e-9 to 5e-3 was 30 times further off. Pairs added in FP64
+// node by node: 254 us a call on the 256^3 pack in FP32; 152 us so, as with the carried pair.) Then
+// a warp shuffle tree, one partial per block and a fixed-order single-block pass. No atomics, so the result depends only
+// on the launch shape, which is fixed per context. What is the same at every node (half a uniform
+// force, and the 1 of rho = 1 + sum h) enters the final sum once: subtracted per node or thread
+// its rounding is the same everywhere and adds up. The half force of a field is summed per warp.
 constexpr int RED_THREADS = MOM_THREADS;
-constexpr int RED_FLUSH = 4;
+constexpr int RED_FLUSH = 16;
+struct TripleMoments {
+    float s[4], e[4], ee[4];
+    __device__ __forceinline__ void add(const PairMoments& m) {
+        for (int c = 0; c < 4; c++) {
+            const dfl t = two_sum(s[c], m.s[c]), u = two_sum(e[c], t.l), v = two_sum(u.h, m.e[c]);
+            s[c] = t.h;
+            e[c] = v.h;
+            ee[c] = __fadd_rn(ee[c], __fadd_rn(u.l, v.l));
+        }
+    }
+    // far from the largest FP32 number, which a sum of RED_FLUSH moments then cannot reach
+    __device__ __forceinline__ bool moderate() const {
+        return fmaxf(fmaxf(fabsf(s[0]), fabsf(s[1])), fmaxf(fabsf(s[2]), fabsf(s[3]))) < 0x1p100f;
+    }
+};
 
 // resident CTAs per SM, and the grid: the 128-bit sums of FP64 storage need the registers
 template <int DT> constexpr int red_ctas() { return DT == LBM_F64 ? 3 : 4; }
@@ -526,9 +545,9 @@ __global__ void __launch_bounds__(RED_THREADS, red_ctas<DT>()) k_reduce(const ty
                                                         const typename Store<DT>::R* __restrict__ gfield_c,
                                                         int64_t n_groups, StepParams p,
                                                         double* __restrict__ partials) {
-    const int t = threadIdx.x;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0}, fx = 0.0;
-    int64_t nodes = 0;
+    __shared__ double sh[RED_THREADS / 32][4], sh_fx[RED_THREADS / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    double fx = 0.0;
     if constexpr (DT == LBM_F64) {
         __int128 sum[4] = {0, 0, 0, 0};
         bool nonfinite = false;
@@ -540,62 +559,79 @@ __global__ void __launch_bounds__(RED_THREADS, red_ctas<DT>()) k_reduce(const ty
             for (int a = 0; a < 3; a++) sum[1 + a] += m.j[a];
             nonfinite |= m.nonfinite;
             if (gfield_c) fx += gfield_c[h.z + t];
-            nodes++;
         }
-        for (int c = 0; c < 4; c++) {
+        nonfinite = __any_sync(0xffffffffu, nonfinite);
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const uint64_t lo = __shfl_down_sync(0xffffffffu, (uint64_t)sum[c], o);
+                const uint64_t hi = __shfl_down_sync(0xffffffffu, (uint64_t)(sum[c] >> 64), o);
+                sum[c] += (__int128)(((unsigned __int128)hi << 64) | lo);
+            }
+        for (int c = 0; c < 4 && lane == 0; c++) {
             // of the magnitude, so that a small negative sum has no large low word
             const bool neg = sum[c] < 0;
             const unsigned __int128 a = neg ? -(unsigned __int128)sum[c] : (unsigned __int128)sum[c];
             const double hi = __ull2double_rn((uint64_t)(a >> 64)), lo = __ull2double_rn((uint64_t)a);
             const double v = __fma_rn(hi, 18446744073709551616.0, lo) * (1.0 / (double)(1ull << FIX_SHIFT));
-            acc[c] = nonfinite ? __longlong_as_double(0x7ff8000000000000ll) : neg ? -v : v;
+            sh[warp][c] = nonfinite ? __longlong_as_double(0x7ff8000000000000ll) : neg ? -v : v;
         }
     } else {
-        PairMoments m = {};
+        TripleMoments m = {};
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
         int held = 0;
         auto flush = [&]() {
-            for (int c = 0; c < 4; c++) {
-                acc[c] += (double)m.s[c];
-                acc[c] += (double)m.e[c];
-            }
+            for (int c = 0; c < 4; c++) acc[c] += (double)m.s[c] + ((double)m.e[c] + (double)m.ee[c]);
             m = {};
             held = 0;
         };
         for (int64_t g = blockIdx.x; g < n_groups; g += gridDim.x) {
             const int4 h = groups[g];
             if (t >= h.w) continue;
-            add_node_moments<DT>(f + (p.sg0 + g) * (Q * GROUP_LANES) + t, m);
-            if (++held == RED_FLUSH) flush();
+            PairMoments node = {};
+            add_node_moments<DT>(f + (p.sg0 + g) * (Q * GROUP_LANES) + t, node);
+            m.add(node);
+            if (++held == RED_FLUSH || !m.moderate()) flush();
             if (gfield_c) fx += (double)gfield_c[h.z + t];
-            nodes++;
         }
-        flush();
-        acc[0] += (double)nodes;   // rho = 1 + sum h
+        if (held) flush();
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            double v = acc[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) sh[warp][c] = v;
+        }
     }
-    acc[1] -= 0.5 * (gfield_c ? fx : (double)nodes * p.g[0]);
-    acc[2] -= 0.5 * ((double)nodes * p.g[1]);
-    acc[3] -= 0.5 * ((double)nodes * p.g[2]);
-    __shared__ double sh[RED_THREADS / 32][4];
-    const int lane = t & 31, warp = t >> 5;
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        double v = acc[c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[warp][c] = v;
+    if (gfield_c) {
+        for (int o = 16; o > 0; o >>= 1) fx += __shfl_down_sync(0xffffffffu, fx, o);
+        if (lane == 0) sh_fx[warp] = fx;
     }
     __syncthreads();
     if (t < 4) {
         double v = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; w++) v += sh[w][t];
+        for (int w = 0; w < RED_THREADS / 32; w++) v += gfield_c && t == 1 ? sh[w][t] - 0.5 * sh_fx[w] : sh[w][t];
         partials[blockIdx.x * 4 + t] = v;
     }
 }
 
-// Fixed-order sum of the blocks' partials: 64 threads per component add every 64th partial,
-// then a shuffle tree over the eight of a warp and the eight warps in order.
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __restrict__ partials, int nb,
-                                                              double* __restrict__ out) {
+// a + b = s + e exactly, in FP64 (two_sum)
+__device__ __forceinline__ void add_exact(double& s, double& e, double b) {
+    const double t = __dadd_rn(s, b), bb = __dadd_rn(t, -s);
+    e = __dadd_rn(e, __dadd_rn(__dadd_rn(s, __dadd_rn(bb, -t)), __dadd_rn(b, -bb)));
+    s = t;
+}
+
+// Fixed-order sum of the blocks' partials: 64 threads per component add every 64th partial, then
+// a shuffle tree over the eight of a warp and one over the warps, which keeps the rounding errors,
+// as does the addition of n_nodes times `each`, the part that every node has alike. (With plain
+// additions, eight in a row at the end, the mass was off by 1.0 half units in the last place, rms.)
+struct NodeConst {
+    double each[4];
+};
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __restrict__ partials, int nb, double n_nodes,
+                                                              NodeConst k, double* __restrict__ out) {
     __shared__ double sh[RED_THREADS / 32][4];
     const int c = threadIdx.x & 3;
     double v = 0.0;
@@ -604,12 +640,24 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __re
     for (int o = 16; o >= 4; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) < 4) sh[threadIdx.x >> 5][c] = v;
     __syncthreads();
-    if (threadIdx.x < 4) {
-        double s = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; w++) s += sh[w][threadIdx.x];
-        out[threadIdx.x] = s;
+    if (threadIdx.x < 32) {
+        double s = sh[threadIdx.x >> 2][c], e = 0.0;
+#pragma unroll
+        for (int o = 16; o >= 4; o >>= 1) {
+            const double s2 = __shfl_down_sync(0xffffffffu, s, o), e2 = __shfl_down_sync(0xffffffffu, e, o);
+            e += e2;
+            add_exact(s, e, s2);
+        }
+        if (threadIdx.x < 4) {
+            const double each = c == 0 ? k.each[0] : c == 1 ? k.each[1] : c == 2 ? k.each[2] : k.each[3];
+            const double all = __dmul_rn(n_nodes, each);
+            e += __fma_rn(n_nodes, each, -all);
+            add_exact(s, e, all);
+            out[c] = s + e;
+        }
     }
 }
+static_assert(RED_THREADS / 32 == 8, "the last tree is over eight warps");
 
 int reduce_blocks(int64_t n_tiles) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((n_tiles * SLOTS + RED_THREADS - 1) / RED_THREADS, 152 * 4));
@@ -631,7 +679,9 @@ template <int DT> static int reduce_dt(lbm_ctx* c) {
 cudaError_t launch_reduce(lbm_ctx* c, double* d_out) {
     const int nb = c->dtype == LBM_F64 ? reduce_dt<LBM_F64>(c) : c->dtype == LBM_F32 ? reduce_dt<LBM_F32>(c)
                                                                                      : reduce_dt<LBM_F16S>(c);
-    k_reduce_final<<<1, RED_THREADS, 0, c->stream>>>(c->partials, nb, d_out);
+    const NodeConst k = {{c->dtype == LBM_F64 ? 0.0 : 1.0, c->gfield ? 0.0 : -0.5 * c->p.g[0], -0.5 * c->p.g[1],
+                          -0.5 * c->p.g[2]}};
+    k_reduce_final<<<1, RED_THREADS, 0, c->stream>>>(c->partials, nb, (double)c->n_own_nonsolid, k, d_out);
     return cudaGetLastError();
 }
 

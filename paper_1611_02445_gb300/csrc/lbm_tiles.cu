@@ -514,10 +514,11 @@ __device__ __forceinline__ void add_node_moments(const typename Store<DT>::T* __
 // carried over four nodes lost the last bits of small populations beside large ones: the
 // momentum of FP32 populations from 1e-9 to 5e-3 was 30 times further off. Pairs added in FP64
 // node by node: 254 us a call on the 256^3 pack in FP32; 152 us so, as with the carried pair.) Then
-// a warp shuffle tree, one partial per block and a fixed-order single-block pass. No atomics, so the result depends only
-// on the launch shape, which is fixed per context. What is the same at every node (half a uniform
-// force, and the 1 of rho = 1 + sum h) enters the final sum once: subtracted per node or thread
-// its rounding is the same everywhere and adds up. The half force of a field is summed per warp.
+// a warp shuffle tree, one partial per block and a fixed-order single-block pass. No atomics, so
+// the result depends only on the launch shape, which is fixed per context. What is the same at
+// every node (half a uniform force, and the 1 of rho = 1 + sum h) enters the final sum once:
+// subtracted per node or thread its rounding is the same everywhere and adds up. The half force
+// of a field is summed per warp.
 constexpr int RED_THREADS = MOM_THREADS;
 constexpr int RED_FLUSH = 16;
 struct TripleMoments {
@@ -786,9 +787,19 @@ __global__ void __launch_bounds__(MOM_THREADS, 4) k_macro(const typename Store<D
                 wide();
             }
         } else {
-            dfl r, j[3], half[3];
-            if constexpr (DT == LBM_F64) half[0] = gfield_c ? df_from_double(gfield_c[hd.z + t]) : p.dfc.Fx;
-            else half[0] = gfield_c ? df_make(gfield_c[hd.z + t], 0.f) : p.dfc.Fx;
+            dfl r, j[3], half[3] = {p.dfc.Fx, {}, {}};
+            bool pair_force = true;
+            if constexpr (DT == LBM_F64) {
+                if (gfield_c) {
+                    const double Fx = gfield_c[hd.z + t];
+                    half[0] = df_from_double(Fx);
+                    // the range of that conversion: [2^-60, 2), or 0
+                    const uint64_t e = bits_of(Fx) << 1;
+                    pair_force = e == 0 || (uint32_t)(e >> 53) - 963u <= 60u;
+                }
+            } else if (gfield_c) {
+                half[0] = df_make(gfield_c[hd.z + t], 0.f);
+            }
             half[0] = df_scale2(half[0], 0.5f);
             half[1] = df_scale2(p.dfc.Fy, 0.5f);
             half[2] = df_scale2(p.dfc.Fz, 0.5f);
@@ -797,7 +808,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 4) k_macro(const typename Store<D
                 r = df_from_fix(fm.r);
                 for (int a = 0; a < 3; a++) j[a] = df_from_fix(fm.j[a]);
                 o = fields_of(r, j, half, inc, ok);
-                ok = ok && !fm.nonfinite;
+                ok = ok && !fm.nonfinite && pair_force;
             } else {
                 r = df_add_dom(df_make(1.0f, 0.0f), df_make(pm.s[0], pm.e[0]));
                 for (int a = 0; a < 3; a++) j[a] = df_make(pm.s[1 + a], pm.e[1 + a]);

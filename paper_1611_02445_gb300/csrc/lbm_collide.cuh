@@ -306,52 +306,9 @@ __device__ __forceinline__ void relax_products(float v[Q], const float ve[Q], co
 // share their terms, instead of two 19 x 19 products each way. FP32, cavity 128^3: 108 -> 69 us
 // a step (the products issued 77 % of cycles), and 1.6e-7 -> 1e-7 off FP64.
 //
-// Non-equilibrium moments that hold no multiple of the density, from sums and differences of
-// the populations (or of h: the weights' contribution to each is zero), in R or in 64-bit
-// fixed point (T): n1 = (e + 11 rho) / 19, n2 = eps - 3 rho, nq = q.
-template <typename T> struct MrtMoments {
-    T rho, j[3], n1, n2, nq[3], pxx, pixx, pww, piww, pxy, pyz, pxz, m[3];
-};
-template <typename T> __device__ __forceinline__ MrtMoments<T> mrt_moments(const T v[Q]) {
-    const T sx = v[1] + v[3], sy = v[2] + v[4], sz = v[5] + v[6];
-    const T a1 = v[7] + v[9], a2 = v[8] + v[10], b1 = v[11] + v[14], b2 = v[12] + v[13], c1 = v[15] + v[18],
-            c2 = v[16] + v[17];
-    const T dx = v[1] - v[3], dy = v[2] - v[4], dz = v[5] - v[6];
-    const T d79 = v[7] - v[9], d810 = v[8] - v[10], d1114 = v[11] - v[14], d1213 = v[12] - v[13],
-            d1518 = v[15] - v[18], d1617 = v[16] - v[17];
-    const T pxy = a1 + a2, pxz = b1 + b2, pyz = c1 + c2;
-    const T ax = (sx + sy) + sz, dg = (pxy + pxz) + pyz;
-    MrtMoments<T> o;
-    o.rho = (v[0] + ax) + dg;
-    o.n1 = dg - v[0];
-    o.n2 = T(9) * v[0] - T(7) * ax - T(2) * dg;
-    const T ex = T(2) * sx - (sy + sz), ed = (pxy + pxz) - T(2) * pyz;
-    const T wx = sy - sz, wd = pxy - pxz;
-    o.pxx = ed + ex;
-    o.pixx = ed - T(2) * ex;
-    o.pww = wd + wx;
-    o.piww = wd - T(2) * wx;
-    o.pxy = a1 - a2;
-    o.pyz = c1 - c2;
-    o.pxz = b1 - b2;
-    // the two diagonal planes of each axis
-    const T x1 = d79 - d810, x2 = d1114 + d1213, y1 = d1518 + d1617, y2 = d79 + d810, z1 = d1114 - d1213,
-            z2 = d1518 - d1617;
-    const T xs = x1 + x2, ys = y1 + y2, zs = z1 + z2;
-    o.j[0] = dx + xs;
-    o.j[1] = dy + ys;
-    o.j[2] = dz + zs;
-    o.nq[0] = xs - T(4) * dx;
-    o.nq[1] = ys - T(4) * dy;
-    o.nq[2] = zs - T(4) * dz;
-    o.m[0] = x1 - x2;
-    o.m[1] = y1 - y2;
-    o.m[2] = z1 - z2;
-    return o;
-}
-
-// v += M^T t from the moments, J and u. p.mrt_s and p.mrt_b hold the rates with |M_k|^2 and the
-// factors above folded in (StepParams). XF: the force has no y or z component.
+// v += M^T t from the moments (MrtMoments, lbm_collide_df.cuh), J and u. p.mrt_s and p.mrt_b hold
+// the rates with |M_k|^2 and the factors above folded in (StepParams). XF: the force has no y or
+// z component.
 template <typename R, bool XF>
 __device__ __forceinline__ void mrt_relax(R v[Q], const MrtMoments<R>& n, const R J[3], const R u[3], const R F[3],
                                           const StepParams& p) {
@@ -421,20 +378,13 @@ __device__ __forceinline__ void collide_mrt(R v[Q], const StepParams& p, R Fx, R
 // the relaxation and M^T t, about 150 operations a node, and bounds the step (2 lanes per SM).
 // Porous 128^3 (0.73 M nodes): 1.57 ms a step with 19 x 19 products in FP64 (about 900
 // operations), 0.36 ms with the moments of collide_mrt, 0.25 ms so, 0.21 ms for a force along x
-// (XF). The velocity after 15 steps
-// is off by 1.8e-13 relative to long double (9.5e-13 with the products).
-// For populations in [2^-6, 2) and a density below 3: no moment then leaves 64 bits (the
-// largest is eps - 3 rho, below 27 of the 32 that fit; the sum of 19 such values is below 38,
-// and one of 32 or more would come out negative). Any other node is left as it is and
-// refused: it takes FP64 throughout.
+// (XF). The velocity after 15 steps is off by 1.8e-13 relative to long double (9.5e-13 with the
+// products).
+// A node that mrt_fix_moments refuses is left as it is: it takes FP64 throughout.
 template <bool XF>
 __device__ __forceinline__ bool collide_mrt_fix(double v[Q], const StepParams& p, double Fx) {
-    int64_t q[Q];
-    bool bad = false;
-#pragma unroll
-    for (int i = 0; i < Q; i++) q[i] = fix_from_double_fast(v[i], bad, 6u);
-    const MrtMoments<int64_t> m = mrt_moments(q);
-    if (bad || m.rho <= 0 || m.rho >= (3ll << FIX_SHIFT)) return false;
+    MrtMoments<int64_t> m;
+    if (!mrt_fix_moments(v, m)) return false;
     MrtMoments<double> n;
     n.rho = fix_to_double(m.rho);
     n.n1 = fix_to_double(m.n1);

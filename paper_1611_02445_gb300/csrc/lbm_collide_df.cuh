@@ -155,16 +155,20 @@ LBM_DF_HD void df_pair(double& a, double& b, const DFConst& K, int k, dfl cj, bo
 }
 
 // Density and momentum from the 19 fixed-point populations, through the pair sums and
-// differences of opposite directions.
-LBM_DF_HD void fix_moments(const int64_t q[19], int64_t& rho, int64_t& jx, int64_t& jy, int64_t& jz) {
-    const int64_t s13 = q[1] + q[3], s24 = q[2] + q[4], s56 = q[5] + q[6], s79 = q[7] + q[9], s810 = q[8] + q[10];
-    const int64_t s1114 = q[11] + q[14], s1213 = q[12] + q[13], s1518 = q[15] + q[18], s1617 = q[16] + q[17];
-    const int64_t d13 = q[1] - q[3], d24 = q[2] - q[4], d56 = q[5] - q[6], d79 = q[7] - q[9], d810 = q[8] - q[10];
-    const int64_t d1114 = q[11] - q[14], d1213 = q[12] - q[13], d1518 = q[15] - q[18], d1617 = q[16] - q[17];
-    rho = q[0] + s13 + s24 + s56 + s79 + s810 + s1114 + s1213 + s1518 + s1617;
-    jx = d13 + d79 - d810 + d1114 + d1213;
-    jy = d24 + d79 + d810 + d1518 + d1617;
-    jz = d56 + d1114 - d1213 + d1518 - d1617;
+// differences of opposite directions; in unsigned arithmetic, since the caller may hold values that
+// it will not use and whose sums overflow.
+LBM_DF_HD void fix_moments(const int64_t f[19], int64_t& rho, int64_t& jx, int64_t& jy, int64_t& jz) {
+    uint64_t q[19];
+#pragma unroll
+    for (int i = 0; i < 19; i++) q[i] = (uint64_t)f[i];
+    const uint64_t s13 = q[1] + q[3], s24 = q[2] + q[4], s56 = q[5] + q[6], s79 = q[7] + q[9], s810 = q[8] + q[10];
+    const uint64_t s1114 = q[11] + q[14], s1213 = q[12] + q[13], s1518 = q[15] + q[18], s1617 = q[16] + q[17];
+    const uint64_t d13 = q[1] - q[3], d24 = q[2] - q[4], d56 = q[5] - q[6], d79 = q[7] - q[9], d810 = q[8] - q[10];
+    const uint64_t d1114 = q[11] - q[14], d1213 = q[12] - q[13], d1518 = q[15] - q[18], d1617 = q[16] - q[17];
+    rho = (int64_t)(q[0] + s13 + s24 + s56 + s79 + s810 + s1114 + s1213 + s1518 + s1617);
+    jx = (int64_t)(d13 + d79 - d810 + d1114 + d1213);
+    jy = (int64_t)(d24 + d79 + d810 + d1518 + d1617);
+    jz = (int64_t)(d56 + d1114 - d1213 + d1518 - d1617);
 }
 
 // Exact moments of a node in 64-bit fixed point. Populations in [2^-6, 16), every one of a
@@ -183,6 +187,81 @@ LBM_DF_HD void node_moments(const double f[19], int64_t& rho, int64_t& jx, int64
         for (int i = 0; i < 19; i++) q[i] = fix_from_double_cvt(f[i]);
         fix_moments(q, rho, jx, jy, jz);
     }
+}
+
+// Moments of the MRT collision (mrt_row in lbm_collide.cuh): the density, the momentum and
+// non-equilibrium moments that hold no multiple of the density, from sums and differences of
+// the populations (or of h: the weights' contribution to each is zero), in floating point or in
+// unsigned 64-bit fixed point (T), where a sum out of range wraps: n1 = (e + 11 rho) / 19,
+// n2 = eps - 3 rho, nq = q.
+template <typename T> struct MrtMoments {
+    T rho, j[3], n1, n2, nq[3], pxx, pixx, pww, piww, pxy, pyz, pxz, m[3];
+};
+template <typename T> LBM_DF_HD MrtMoments<T> mrt_moments(const T v[19]) {
+    const T sx = v[1] + v[3], sy = v[2] + v[4], sz = v[5] + v[6];
+    const T a1 = v[7] + v[9], a2 = v[8] + v[10], b1 = v[11] + v[14], b2 = v[12] + v[13], c1 = v[15] + v[18],
+            c2 = v[16] + v[17];
+    const T dx = v[1] - v[3], dy = v[2] - v[4], dz = v[5] - v[6];
+    const T d79 = v[7] - v[9], d810 = v[8] - v[10], d1114 = v[11] - v[14], d1213 = v[12] - v[13],
+            d1518 = v[15] - v[18], d1617 = v[16] - v[17];
+    const T pxy = a1 + a2, pxz = b1 + b2, pyz = c1 + c2;
+    const T ax = (sx + sy) + sz, dg = (pxy + pxz) + pyz;
+    MrtMoments<T> o;
+    o.rho = (v[0] + ax) + dg;
+    o.n1 = dg - v[0];
+    o.n2 = T(9) * v[0] - T(7) * ax - T(2) * dg;
+    const T ex = T(2) * sx - (sy + sz), ed = (pxy + pxz) - T(2) * pyz;
+    const T wx = sy - sz, wd = pxy - pxz;
+    o.pxx = ed + ex;
+    o.pixx = ed - T(2) * ex;
+    o.pww = wd + wx;
+    o.piww = wd - T(2) * wx;
+    o.pxy = a1 - a2;
+    o.pyz = c1 - c2;
+    o.pxz = b1 - b2;
+    // the two diagonal planes of each axis
+    const T x1 = d79 - d810, x2 = d1114 + d1213, y1 = d1518 + d1617, y2 = d79 + d810, z1 = d1114 - d1213,
+            z2 = d1518 - d1617;
+    const T xs = x1 + x2, ys = y1 + y2, zs = z1 + z2;
+    o.j[0] = dx + xs;
+    o.j[1] = dy + ys;
+    o.j[2] = dz + zs;
+    o.nq[0] = xs - T(4) * dx;
+    o.nq[1] = ys - T(4) * dy;
+    o.nq[2] = zs - T(4) * dz;
+    o.m[0] = x1 - x2;
+    o.m[1] = y1 - y2;
+    o.m[2] = z1 - z2;
+    return o;
+}
+
+// The same from FP64 populations, exactly, for populations in [2^-6, 2) and a density below 3: no
+// moment then leaves 64 bits (the largest is eps - 3 rho, below 27 of the 32 that fit; the
+// density of 19 such values is below 38, of the 64 that the unsigned sum holds). Any other node is
+// refused.
+LBM_DF_HD bool mrt_fix_moments(const double v[19], MrtMoments<int64_t>& m) {
+    uint64_t q[19];
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < 19; i++) q[i] = (uint64_t)fix_from_double_fast(v[i], bad, 6u);
+    const MrtMoments<uint64_t> n = mrt_moments(q);
+    if (bad || n.rho >= (3ull << FIX_SHIFT)) return false;
+    m.rho = (int64_t)n.rho;
+    m.n1 = (int64_t)n.n1;
+    m.n2 = (int64_t)n.n2;
+    m.pxx = (int64_t)n.pxx;
+    m.pixx = (int64_t)n.pixx;
+    m.pww = (int64_t)n.pww;
+    m.piww = (int64_t)n.piww;
+    m.pxy = (int64_t)n.pxy;
+    m.pyz = (int64_t)n.pyz;
+    m.pxz = (int64_t)n.pxz;
+    for (int a = 0; a < 3; a++) {
+        m.j[a] = (int64_t)n.j[a];
+        m.nq[a] = (int64_t)n.nq[a];
+        m.m[a] = (int64_t)n.m[a];
+    }
+    return true;
 }
 
 // f: the 19 gathered populations of a fluid node, replaced by the post-collision ones.

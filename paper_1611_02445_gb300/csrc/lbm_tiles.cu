@@ -469,17 +469,19 @@ __device__ __forceinline__ FixMoments fix_node_moments(const double* __restrict_
     for (int i = 0; i < Q; i++) q[i] = fix_from_double_fast(f[i * GROUP_LANES], bad);
     fix_moments(q, m.r, m.j[0], m.j[1], m.j[2]);
     if (bad) {
-        m.r = m.j[0] = m.j[1] = m.j[2] = 0;
+        uint64_t r = 0, j[3] = {0, 0, 0};   // unsigned: values of 16 and more may wrap
 #pragma unroll 1
         for (int i = 0; i < Q; i++) {
             const double v = f[i * GROUP_LANES];
             m.nonfinite |= (~bits_of(v) & 0x7ff0000000000000ull) == 0;
-            const int64_t w = fix_from_double(v);
-            m.r += w;
-            m.j[0] += cx(i) * w;
-            m.j[1] += cy(i) * w;
-            m.j[2] += cz(i) * w;
+            const uint64_t w = (uint64_t)fix_from_double(v);
+            r += w;
+            j[0] += (uint64_t)(int64_t)cx(i) * w;
+            j[1] += (uint64_t)(int64_t)cy(i) * w;
+            j[2] += (uint64_t)(int64_t)cz(i) * w;
         }
+        m.r = (int64_t)r;
+        for (int a = 0; a < 3; a++) m.j[a] = (int64_t)j[a];
     }
     return m;
 }

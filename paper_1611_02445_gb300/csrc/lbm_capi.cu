@@ -508,8 +508,8 @@ static lbm_status create_impl(const uint8_t* node_type, int on_device, int nx, i
         const size_t copy_bytes = (size_t)sgroups * lbm::Q * lbm::GROUP_LANES * lbm::dtype_size(dtype);
         LBM_CREATE_CUDA(lbm::dmalloc(&c->f[0], std::max<size_t>(copy_bytes, 16)));
         LBM_CREATE_CUDA(lbm::dmalloc(&c->f[1], std::max<size_t>(copy_bytes, 16)));
-        // the padding lanes of the groups are never read or written: zero, so that a saved
-        // state depends on the populations alone
+        // the padding lanes of the groups are never written, nor used where they are read along with
+        // their neighbours: zero, so that a saved state depends on the populations alone
         LBM_CREATE_CUDA(cudaMemsetAsync(c->f[0], 0, copy_bytes, c->stream));
         LBM_CREATE_CUDA(cudaMemsetAsync(c->f[1], 0, copy_bytes, c->stream));
         {

@@ -87,6 +87,7 @@ constexpr int GROUP_MAX_NODES = 256;       // work-group size of the 4-byte-or-s
 constexpr int GROUP_MAX_NODES_F64 = 256;   // and of FP64 storage (see the step kernel's CTA shape)
 constexpr int GROUP_LANES = 256;           // lanes of a storage group: the length of its data blocks
 constexpr int GROUP_MAX_IMPORTS = 1536;    // imports of a work group the FP16 step can stage
+constexpr int THIN_NODES = 48;             // nodes a work group below which the FP16 step copies parts of blocks
 constexpr int FLAG_HAS_BC = 1;
 // F16S storage scale: h is stored as half(h * 2^12), so |h| in [1.5e-8, 16] is normal.
 constexpr float F16_SCALE = 4096.0f;

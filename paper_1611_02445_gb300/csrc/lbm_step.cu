@@ -469,6 +469,10 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
 // 66 % of cycles; the lists cost 32 bytes a node more than the ranks, which FP16, at 44 % of
 // the DRAM rate, has room for. (FP32 and FP64 are nearer to the DRAM rate and keep the pulls.)
 // Measured: 188 us (25.1 -> 31.2 GLUPS); 190^3 cavity 1.24 times, 32^3 channel 1.05 times as fast.
+// THIN copies only the part of the blocks that holds nodes. With whole blocks the step was 1 % slower
+// than node-by-node pulls on tubes one node wide (32 nodes a group: 48.0 against 47.5 us, 46.7 so);
+// at 46 nodes a group it is as fast either way (105.7 us, a random box of 256^3 nodes), above
+// that looking at the count costs 0.1 to 0.5 %.
 constexpr int RUN_BYTES = Q * GROUP_LANES * 2;
 constexpr int RUN_CHUNKS = RUN_BYTES / 16;
 struct RunSmem {
@@ -483,7 +487,7 @@ struct RunSmem {
     float gf[GROUP_LANES];                              // last (see StepSmem)
 };
 
-template <bool VAR, int MODE, bool GEN>
+template <bool VAR, int MODE, bool GEN, bool THIN>
 __global__ void __launch_bounds__(GROUP_LANES, 4)
 k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __restrict__ groups,
            const int2* __restrict__ imports, const uint32_t* __restrict__ entries, const uint4* __restrict__ fsrc,
@@ -515,7 +519,9 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
         if (g >= n_groups) return;
         unsigned char* d = sm.data[it & 1];
         const char* run = reinterpret_cast<const char*>(A + (p.sg0 + g) * (Q * GROUP_LANES));
-        for (int k = t; k < RUN_CHUNKS; k += GROUP_LANES) cp_async16(d + 16 * k, run + 16 * k);
+        // a piece is 8 lanes, and a thread's pieces lie at the same place of their blocks
+        if (!THIN || 8 * (t % (GROUP_LANES / 8)) < header(it).w)
+            for (int k = t; k < RUN_CHUNKS; k += GROUP_LANES) cp_async16(d + 16 * k, run + 16 * k);
         if (MODE == STEP_RW) return;
         const int n = sm.imp[it & 3].y;
         for (int k = t; 4 * k < n; k += GROUP_LANES) {
@@ -636,7 +642,7 @@ static int step_grid(int64_t n_groups, bool with_gf) {
 }
 
 // Persistent grid of the FP16 step on staged runs.
-template <bool VAR, int MODE, bool GEN>
+template <bool VAR, int MODE, bool GEN, bool THIN>
 static int run_grid(int64_t n_groups, bool with_gf) {
     static int per_sm[2] = {-1, -1}, n_sm = 0;
     int& ps = per_sm[with_gf ? 1 : 0];
@@ -644,24 +650,38 @@ static int run_grid(int64_t n_groups, bool with_gf) {
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RunSmem));
-        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_step_run<VAR, MODE, GEN>, GROUP_LANES,
+        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN, THIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RunSmem));
+        cudaFuncSetAttribute(k_step_run<VAR, MODE, GEN, THIN>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_step_run<VAR, MODE, GEN, THIN>, GROUP_LANES,
                                                       with_gf ? sizeof(RunSmem) : offsetof(RunSmem, gf));
         ps = std::max(1, std::min(ps, 4));
     }
     return (int)std::max<int64_t>(1, std::min<int64_t>(n_groups, (int64_t)ps * n_sm));
 }
 
-template <bool VAR, int MODE, bool GEN>
-static cudaError_t launch_run(lbm_ctx* c, const void* A, void* B, bool chained) {
+template <bool VAR, int MODE, bool GEN, bool THIN>
+static cudaError_t launch_run_of(lbm_ctx* c, const void* A, void* B, bool chained) {
     const bool with_gf = c->gfield != nullptr;
     const int from = A == c->f[0] ? 0 : 1;
-    return launch_chained(k_step_run<VAR, MODE, GEN>, (unsigned)run_grid<VAR, MODE, GEN>(c->n_groups, with_gf),
+    return launch_chained(k_step_run<VAR, MODE, GEN, THIN>, (unsigned)run_grid<VAR, MODE, GEN, THIN>(c->n_groups, with_gf),
                           (unsigned)GROUP_LANES, with_gf ? sizeof(RunSmem) : offsetof(RunSmem, gf), c->stream, chained,
                           (const __half*)A, (__half*)B, c->groups, c->imports, c->entries, c->fsrc, c->fsrc8, c->fword,
                           with_gf ? (const float*)c->gfield_c : nullptr, c->n_groups, c->p,
                           c->seed ? c->seed + from : nullptr, c->seed ? c->seed + (1 - from) : nullptr);
+}
+
+// Work groups of fewer than THIN_NODES nodes on average.
+static bool thin_groups(const lbm_ctx* c) { return c->n_own_nonsolid < THIN_NODES * c->n_groups; }
+
+template <bool VAR, int MODE, bool GEN>
+static cudaError_t launch_run(lbm_ctx* c, const void* A, void* B, bool chained) {
+    return thin_groups(c) ? launch_run_of<VAR, MODE, GEN, true>(c, A, B, chained)
+                          : launch_run_of<VAR, MODE, GEN, false>(c, A, B, chained);
+}
+
+template <bool VAR, bool GEN> static void prepare_run(lbm_ctx* c) {
+    if (thin_groups(c)) run_grid<VAR, STEP_FULL, GEN, true>(1, c->gfield != nullptr);
+    else run_grid<VAR, STEP_FULL, GEN, false>(1, c->gfield != nullptr);
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
@@ -758,8 +778,8 @@ static void prepare_model(lbm_ctx* c) {
         case LBM_F32: prepare_dt<LBM_F32, false, GEN, false>(c); break;
         default:
             if (c->fsrc) {
-                if (c->sr) run_grid<true, STEP_FULL, GEN>(1, c->gfield != nullptr);
-                else run_grid<false, STEP_FULL, GEN>(1, c->gfield != nullptr);
+                if (c->sr) prepare_run<true, GEN>(c);
+                else prepare_run<false, GEN>(c);
                 break;
             }
             if (c->sr) prepare_dt<LBM_F16S, true, GEN, false>(c);

@@ -510,7 +510,7 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
     };
     // the imports' source words: thread t reads and later uses entries 4 t ... 4 t + 3 (+ 1024)
     const auto issue_entries = [&](int it) {
-        if (MODE == STEP_RW || g0 + it * G >= n_groups) return;
+        if (g0 + it * G >= n_groups) return;
         const int2 m = sm.imp[it & 3];
         for (int k = t; 4 * k < m.y; k += GROUP_LANES) cp_async16(&sm.entry[k], entries + m.x + 4 * k);
     };
@@ -522,7 +522,6 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
         // a piece is 8 lanes, and a thread's pieces lie at the same place of their blocks
         if (!THIN || 8 * (t % (GROUP_LANES / 8)) < header(it).w)
             for (int k = t; k < RUN_CHUNKS; k += GROUP_LANES) cp_async16(d + 16 * k, run + 16 * k);
-        if (MODE == STEP_RW) return;
         const int n = sm.imp[it & 3].y;
         for (int k = t; 4 * k < n; k += GROUP_LANES) {
             const uint4 e = sm.entry[k];
@@ -592,7 +591,7 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
 #pragma unroll
         for (int i = 0; i < Q; i++) {
             uint32_t o = (uint32_t)(i * GROUP_LANES + t) * 2u;
-            if (MODE != STEP_RW && i > 0) o = (i & 1) ? off[(i - 1) >> 1] & 0xffffu : off[(i - 1) >> 1] >> 16;
+            if (i > 0) o = (i & 1) ? off[(i - 1) >> 1] & 0xffffu : off[(i - 1) >> 1] >> 16;
             if (!check_ok(o < sizeof(sm.data[0]), CHECK_NEIGHBOUR, (int64_t)h.z + t, p)) o = 0;
             v[i] = to_arith<DT>(*reinterpret_cast<const __half*>(d + o), i);
         }
@@ -673,10 +672,19 @@ static cudaError_t launch_run_of(lbm_ctx* c, const void* A, void* B, bool chaine
 // Work groups of fewer than THIN_NODES nodes on average.
 static bool thin_groups(const lbm_ctx* c) { return c->n_own_nonsolid < THIN_NODES * c->n_groups; }
 
+// Whether the FP16 kernel of a mode runs on staged runs. The read-write-only kernel never does (it
+// needs neither the lists nor the offsets: 256^3 random box with 77 nodes a group 97 us staged, 82 us
+// node by node), the propagation-only kernel not on thin groups (82 and 75 us at 26 nodes a group).
+template <int MODE> static bool takes_runs(const lbm_ctx* c) {
+    return c->fsrc && MODE != STEP_RW && (MODE == STEP_FULL || !thin_groups(c));
+}
+
 template <bool VAR, int MODE, bool GEN>
 static cudaError_t launch_run(lbm_ctx* c, const void* A, void* B, bool chained) {
-    return thin_groups(c) ? launch_run_of<VAR, MODE, GEN, true>(c, A, B, chained)
-                          : launch_run_of<VAR, MODE, GEN, false>(c, A, B, chained);
+    if constexpr (MODE == STEP_FULL) {
+        if (thin_groups(c)) return launch_run_of<VAR, MODE, GEN, true>(c, A, B, chained);
+    }
+    return launch_run_of<VAR, MODE, GEN, false>(c, A, B, chained);
 }
 
 template <bool VAR, bool GEN> static void prepare_run(lbm_ctx* c) {
@@ -746,7 +754,11 @@ static cudaError_t launch_step_model(lbm_ctx* c, const void* A, void* B, bool ch
                                : launch_step_dt<LBM_F64, false, MODE, GEN, false>(c, A, B, chained);
         case LBM_F32: return launch_step_dt<LBM_F32, false, MODE, GEN, false>(c, A, B, chained);
         default:
-            if (c->fsrc) return c->sr ? launch_run<true, MODE, GEN>(c, A, B, chained) : launch_run<false, MODE, GEN>(c, A, B, chained);
+            if constexpr (MODE != STEP_RW) {
+                if (takes_runs<MODE>(c))
+                    return c->sr ? launch_run<true, MODE, GEN>(c, A, B, chained)
+                                 : launch_run<false, MODE, GEN>(c, A, B, chained);
+            }
             return c->sr ? launch_step_dt<LBM_F16S, true, MODE, GEN, false>(c, A, B, chained)
                          : launch_step_dt<LBM_F16S, false, MODE, GEN, false>(c, A, B, chained);
     }
@@ -777,7 +789,7 @@ static void prepare_model(lbm_ctx* c) {
             break;
         case LBM_F32: prepare_dt<LBM_F32, false, GEN, false>(c); break;
         default:
-            if (c->fsrc) {
+            if (takes_runs<STEP_FULL>(c)) {
                 if (c->sr) prepare_run<true, GEN>(c);
                 else prepare_run<false, GEN>(c);
                 break;

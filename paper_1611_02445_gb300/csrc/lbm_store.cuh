@@ -48,9 +48,4 @@ template <> __device__ __forceinline__ double to_store<LBM_F64>(double v, int) {
 template <> __device__ __forceinline__ float to_store<LBM_F32>(float v, int) { return v; }
 template <> __device__ __forceinline__ __half to_store<LBM_F16S>(float v, int) { return __float2half_rn(v * F16_SCALE); }
 
-// per-node x force of the tile-major field
-template <int DT> __device__ __forceinline__ double gfield_at(const void* g, int64_t idx) {
-    return DT == LBM_F64 ? ((const double*)g)[idx] : (double)((const float*)g)[idx];
-}
-
 }  // namespace lbm

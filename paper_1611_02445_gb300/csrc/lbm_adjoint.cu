@@ -306,7 +306,7 @@ k_adjoint(const typename Store<DT>::T* st, const typename Store<DT>::T* sT, cons
             }
         }
     };
-    const int64_t g0 = G - 1 - blockIdx.x;   // as in the step: the CTAs with one group more come last
+    const int64_t g0 = G - 1 - blockIdx.x;   // as in k_step_run: the CTAs with one group more come last
     issue_header(g0, 0);
     issue_header(g0 + G, 1);
     cp_async_commit();
@@ -315,6 +315,7 @@ k_adjoint(const typename Store<DT>::T* st, const typename Store<DT>::T* sT, cons
     issue_meta(g0, 0);
     cp_async_commit();
     grid_wait();   // the tables are constant; from here on the launch before is complete
+    grid_release();
     R tau1 = R(0), tau2 = R(0), err1 = R(0), err2 = R(0);
     int it = 0;
     for (int64_t g = g0; g < nt.n_groups; g += G, it++) {

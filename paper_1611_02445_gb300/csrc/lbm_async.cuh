@@ -6,22 +6,20 @@
 namespace lbm {
 
 // Chained launches. A step launched with `chained` follows another step or adjoint launch of the
-// same call on the stream, and may start while that one's last CTAs still run: its CTAs take
-// the places that become free, load their first headers, records and words (which no launch
+// same call on the stream, or the call's graph replays, and may start before it has ended: its CTAs
+// take the places that are free, load their first headers, records and words (which no launch
 // of the chain writes) and wait in grid_wait() until the launch before has completed and its
 // results are visible. Everything that a launch of the chain writes, or reads from one, comes
 // after grid_wait(), which every CTA executes: so completion is transitive along the chain. A
-// launch lets the next one start only after its own grid_wait(), so no more than two are on the
-// GPU at once and the start of the third (which empties L1) comes after the first has ended;
-// words that share a cache line between CTAs and change from launch to launch are read past L1
-// (__ldcg). The first launch of a call is never chained (the tables may have been written by the
-// work before it). Without the attribute both instructions do nothing.
+// launch lets the next one start (grid_release) only after its own grid_wait(), so no more than
+// two are on the GPU at once and the start of the third (which empties L1) comes after the first
+// has ended; words that share a cache line between CTAs and change from launch to launch are read
+// past L1 (__ldcg). The first launch of a call is never chained (the tables may have been written
+// by the work before it). Without the attribute both instructions do nothing.
 // Against unchained launches of the same kernels, a step: 32^3 channel FP16 4.2 -> 3.1 us, 48^3 pack
 // FP32 4.8 -> 3.7, 96^3 pack FP32 14.7 -> 13.6, 128^3 pack FP64 61 -> 59; 256^3 packs 1 %.
-__device__ __forceinline__ void grid_wait() {
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,

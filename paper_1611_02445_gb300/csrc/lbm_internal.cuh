@@ -161,7 +161,7 @@ struct StepParams {
     double g[3];
     double u_in[3];
     double rho_out;
-    const void* gfield;
+    int reversed, early;   // of one launch (chain_order)
     DFConst dfc;   // constants of the double-float FP64 collision
     DFClosure dfb; // and of its inlet and outlet closures
     // FP32 copies for the 4-byte formats (an FP64 -> FP32 conversion runs on the FP64 pipe)

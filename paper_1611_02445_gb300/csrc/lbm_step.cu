@@ -388,12 +388,9 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StepSmem<DT>& sm = *reinterpret_cast<StepSmem<DT>*>(smem_raw);
     const int64_t G = gridDim.x;   // at most n_groups
-    // The CTAs with one group more than the others are the last ones: a chained launch's CTAs
-    // start in index order on the places that become free, so those with fewer groups follow
-    // each other on the same SMs and so do the others, as the first launch spread them. (FP64
-    // arithmetic throughout: 2.4 ms on the 256^3 pack, where that gains nothing and the reversed
-    // index spills 8 bytes more: 2 446 against 2 415 us, and 1 to 2 % on seven of twelve flows.)
-    const int64_t g0 = DT == LBM_F64 && VAR && !GEN ? blockIdx.x : G - 1 - blockIdx.x;
+    // (FP64 arithmetic throughout: 2.4 ms on the 256^3 pack, where the order gains nothing and its
+    // index spills 8 bytes more: 2 446 against 2 415 us.)
+    const int64_t g0 = !p.reversed || (DT == LBM_F64 && VAR && !GEN) ? blockIdx.x : G - 1 - blockIdx.x;
     const bool has_gf = gfield_c != nullptr;
     // prologue: headers of groups 0..2, meta of groups 0..1, gathers of group 0
     issue_hdr(&sm.hdr[0], g0, n_groups, groups);
@@ -411,6 +408,7 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
     cp_async_wait<1>();
     __syncthreads();
     grid_wait();   // the tables above are constant; from here on the launch before is complete
+    if (p.early) grid_release();
     uint32_t key = 0;
     if (DT == LBM_F16S && VAR) {
         // step counter of the rounding hash: read from this launch's copy, advanced into
@@ -456,6 +454,7 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
             compute_store<DT, VAR, MODE, GEN, XF, INC>(sm, it % META_SLOTS, 0, h, p.sg0 + g, B, p, has_gf, key, gather_next);
         }
     }
+    grid_release();
     cp_async_wait<0>();
 }
 
@@ -500,7 +499,10 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
     constexpr int DT = LBM_F16S;
     const int t = threadIdx.x;
     const int64_t G = gridDim.x;
-    const int64_t g0 = G - 1 - blockIdx.x;   // as in k_step
+    // The CTAs with one group more than the others are the last ones: a chained launch's CTAs
+    // start in index order on the places that become free, so those with fewer groups follow
+    // each other on the same SMs and so do the others, as the first launch spread them.
+    const int64_t g0 = G - 1 - blockIdx.x;
     const bool has_gf = gfield_c != nullptr;
     const auto header = [&](int it) { return group_header<DT>(sm.hdr[it & 3], p); };
     const auto issue_header = [&](int it) {
@@ -564,6 +566,7 @@ k_step_run(const __half* __restrict__ A, __half* __restrict__ B, const int4* __r
     cp_async_commit();
     cp_async_wait<0>();
     grid_wait();   // the tables above are constant; from here on the launch before is complete
+    grid_release();
     uint32_t key = 0;
     if (VAR) {
         // step counter of the rounding hash, as in k_step
@@ -694,18 +697,45 @@ template <bool VAR, bool GEN> static void prepare_run(lbm_ctx* c) {
     else run_grid<VAR, STEP_FULL, GEN, false>(1, c->gfield != nullptr);
 }
 
+// Whether a step lets the next one start at once (early) or when its CTAs finish, and whether CTA b
+// starts with group grid - 1 - b (reversed: the CTAs with one group more than the others then have
+// the highest indices) or with group b.
+// CTAs that start early take whatever places are free and keep them, so the SMs get shares of the
+// next launch that differ from those of an unchained one. Measured over cavities, channels, packs
+// and ducts of 33^3 to 190^3 nodes in FP64 and FP32, a step of 64 in one call against unchained
+// steps (early reversed / late in index order):
+//  - one group per CTA: early, 1.05 to 1.20 times as fast, as long as the next launch finds room for
+//    all its CTAs beside this one or the places are nearly full. Between half and two thirds of the
+//    places the CTAs left over pile up on the SMs that finish first: 0.86 and 0.93 times as fast in
+//    FP64 and FP32, against 1.00 and 1.14 late;
+//  - more than half of the CTAs carry one group more (n / grid = 1.5 to 1.9, 2.5 to 2.9): early
+//    reversed, 1.04 to 1.21 against 1.03 to 1.09. (Not with Zou-He nodes in FP64, whose groups
+//    take longer: 0.92 and 0.97 against 1.02 and 0.99);
+//  - fewer than half do: late in index order, 1.01 to 1.13 against 0.94 to 1.06;
+//  - from five groups a CTA on the shares hardly differ: early.
+static void chain_order(StepParams& p, int64_t n, int64_t grid, int64_t places, bool f64) {
+    if (n <= grid) {
+        p.early = p.reversed = 2 * n <= places || 3 * n >= 2 * places;
+    } else {
+        p.reversed = 2 * (n % grid) > grid && !(f64 && p.bc == LBM_BC_ZOU_HE);
+        p.early = p.reversed || n >= 5 * grid;
+    }
+}
+
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC, bool I32>
 static cudaError_t launch_step_ix(lbm_ctx* c, const void* A, void* B, bool chained) {
     using T = typename Store<DT>::T;
     const bool with_gf = c->gfield != nullptr;
     const int grid = step_grid<DT, VAR, MODE, GEN, XF, INC, I32>(c->n_groups, with_gf);
+    StepParams p = c->p;
+    chain_order(p, c->n_groups, grid, 152 * (int64_t)step_ctas<DT, GEN>(), DT == LBM_F64);
     // the copy read decides which counter is read and which is advanced
     const int from = A == c->f[0] ? 0 : 1;
     const uint32_t* seed_in = c->seed ? c->seed + from : nullptr;
     uint32_t* seed_out = c->seed ? c->seed + (1 - from) : nullptr;
     return launch_chained(k_step<DT, VAR, MODE, GEN, XF, INC, I32>, (unsigned)grid, (unsigned)StepCfg<DT>::THREADS,
                           step_smem<DT>(with_gf), c->stream, chained, (const T*)A, (T*)B, c->groups, c->nrec, c->fword,
-                          c->frank, c->gfield ? c->gfield_c : nullptr, c->n_groups, c->p, seed_in, seed_out);
+                          c->frank, c->gfield ? c->gfield_c : nullptr, c->n_groups, p, seed_in, seed_out);
 }
 
 template <int DT, bool VAR, int MODE, bool GEN, bool XF, bool INC>

@@ -466,10 +466,11 @@ k_step(const typename Store<DT>::T* __restrict__ A, typename Store<DT>::T* __res
 // offsets precomputed at creation (fsrc: own block or import, the half of an import's word, its
 // own opposite direction for a bounced link), with two instructions a value. The per-node
 // pulls of k_step, forming 18 addresses and selecting the half of each staged word, were a
-// third of the FP16 step (233 us on the porous 256^3 pack, 156 us without them), which issues
-// 66 % of cycles; the lists cost 32 bytes a node more than the ranks, which FP16, at 44 % of
-// the DRAM rate, has room for. (FP32 and FP64 are nearer to the DRAM rate and keep the pulls.)
-// Measured: 188 us (25.1 -> 31.2 GLUPS); 190^3 cavity 1.24 times, 32^3 channel 1.05 times as fast.
+// third of the FP16 step (233 us on the porous 256^3 pack, 156 us without them), which issued
+// 66 % of cycles; the lists cost 36 bytes a node more than the ranks, which FP16, at 44 % of
+// the DRAM rate, had room for. (FP32 and FP64 are nearer to the DRAM rate and keep the pulls.)
+// Measured: 190 us (25.1 -> 30.9 GLUPS) at 158 B a node, 0.71 of the DRAM copy rate, and 63 % issue;
+// 190^3 cavity 1.24 times, 32^3 channel 1.05 times as fast.
 // THIN copies only the part of the blocks that holds nodes. With whole blocks the step was 1 % slower
 // than node-by-node pulls on tubes one node wide (32 nodes a group: 48.0 against 47.5 us, 46.7 so);
 // at 46 nodes a group it is as fast either way (105.7 us, a random box of 256^3 nodes), above

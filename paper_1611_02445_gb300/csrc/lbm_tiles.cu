@@ -445,7 +445,7 @@ cudaError_t launch_init(lbm_ctx* c, double rho0, const double u0[3]) {
 // formed with integer (FP64 storage) or FP32 (the other formats) instructions, and FP64 is
 // left for what needs it. Measured against one thread per tile slot with FP64 moments and
 // divisions: k_reduce<F64> 103 -> 45 us on a 160^3 pack (1.4 M nodes, 219 MB: 4.9 TB/s);
-// reduction and FP64 fields together 322 -> 161 us there; the FP32 fields of a 256^3 pack
+// reduction and FP64 fields together 322 -> 159 us there; the FP32 fields of a 256^3 pack
 // (5.9 M nodes) 640 us less. k_macro<F32, float> issues 65 % of cycles (the TwoSums).
 constexpr int MOM_THREADS = GROUP_LANES;   // one thread per lane of a work group
 static_assert(GROUP_MAX_NODES == MOM_THREADS && GROUP_MAX_NODES_F64 == MOM_THREADS, "one thread per lane");

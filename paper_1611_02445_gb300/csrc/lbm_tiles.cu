@@ -585,7 +585,11 @@ __global__ void __launch_bounds__(RED_THREADS, red_ctas<DT>()) k_reduce(const ty
         double acc[4] = {0.0, 0.0, 0.0, 0.0};
         int held = 0;
         auto flush = [&]() {
-            for (int c = 0; c < 4; c++) acc[c] += (double)m.s[c] + ((double)m.e[c] + (double)m.ee[c]);
+            for (int c = 0; c < 4; c++) {
+                double e = (double)m.e[c];
+                if (m.ee[c] != 0.f) e += (double)m.ee[c];   // 0 for a single node: 8 FP64 operations less
+                acc[c] += (double)m.s[c] + e;
+            }
             m = {};
             held = 0;
         };
@@ -619,11 +623,10 @@ __global__ void __launch_bounds__(RED_THREADS, red_ctas<DT>()) k_reduce(const ty
     }
 }
 
-// a + b = s + e exactly, in FP64 (two_sum)
-__device__ __forceinline__ void add_exact(double& s, double& e, double b) {
-    const double t = __dadd_rn(s, b), bb = __dadd_rn(t, -s);
-    e = __dadd_rn(e, __dadd_rn(__dadd_rn(s, __dadd_rn(bb, -t)), __dadd_rn(b, -bb)));
-    s = t;
+// a + b - fl(a + b), exactly (two_sum in FP64)
+__device__ __forceinline__ double sum_error(double a, double b) {
+    const double s = __dadd_rn(a, b), bb = __dadd_rn(s, -a);
+    return __dadd_rn(__dadd_rn(a, __dadd_rn(bb, -s)), __dadd_rn(b, -bb));
 }
 
 // Fixed-order sum of the blocks' partials: 64 threads per component add every 64th partial, then
@@ -644,19 +647,24 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __re
     if ((threadIdx.x & 31) < 4) sh[threadIdx.x >> 5][c] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        double s = sh[threadIdx.x >> 2][c], e = 0.0;
+        // the sums first, then their errors, which depend on the sums alone
+        double s = sh[threadIdx.x >> 2][c], a[3], b[3];
 #pragma unroll
-        for (int o = 16; o >= 4; o >>= 1) {
-            const double s2 = __shfl_down_sync(0xffffffffu, s, o), e2 = __shfl_down_sync(0xffffffffu, e, o);
-            e += e2;
-            add_exact(s, e, s2);
+        for (int k = 0; k < 3; k++) {
+            a[k] = s;
+            b[k] = __shfl_down_sync(0xffffffffu, s, 16 >> k);
+            s = __dadd_rn(a[k], b[k]);
         }
+        double e = sum_error(a[0], b[0]);
+        e += __shfl_down_sync(0xffffffffu, e, 8);
+        e += sum_error(a[1], b[1]);
+        e += __shfl_down_sync(0xffffffffu, e, 4);
+        e += sum_error(a[2], b[2]);
         if (threadIdx.x < 4) {
             const double each = c == 0 ? k.each[0] : c == 1 ? k.each[1] : c == 2 ? k.each[2] : k.each[3];
             const double all = __dmul_rn(n_nodes, each);
             e += __fma_rn(n_nodes, each, -all);
-            add_exact(s, e, all);
-            out[c] = s + e;
+            out[c] = __dadd_rn(s, all) + (e + sum_error(s, all));
         }
     }
 }

@@ -728,10 +728,10 @@ FP64_FLOPS_PER_NODE = 331
 # ncu capture of this workload (dram__bytes_read.sum + dram__bytes_write.sum, the mean of
 # two launches after three warm-up steps), with the hash (step_source_hash) of the library
 # sources they were captured with; the bench reports them only while the sources match.
-TRAFFIC_PER_LAUNCH_256 = {"sources": "716218a1457c00ee",
-                          "f64": 1203237760 + 856190848,
-                          "f32": 686737408 + 416655104,
-                          "f16s": 719982592 + 208483840}
+TRAFFIC_PER_LAUNCH_256 = {"sources": "dfb9044aa73bd9ef",
+                          "f64": 1204476928 + 856307456,
+                          "f32": 686524416 + 416480256,
+                          "f16s": 719437568 + 208505344}
 
 if __name__ == "__main__":
     main()
